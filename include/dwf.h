@@ -374,9 +374,11 @@ long long dwf_launch_count(dwf_handle h);
  * them back row by row (ns and sb must be 0).  ns: slices per thread for the
  * other variants (1, 2 when it divides Ls, 4 for variant 5); sb: sites per
  * CTA.  -1 / 0 select the built-in defaults (FP32: variant 9 where it
- * applies, else 0; FP16: 5; FP64: 0).  Variants differ only in the order of
- * the sums, except 5 (FP16 rounding of the projection) and 10 (products of
- * the TF32 terms).  Numbers 1, 2, 6 and 8 are not used.
+ * applies, else 0; FP16: 5; FP64: a hop on 59-bit fixed-point blocks, for
+ * which dwf_get_hop_config answers 0; any variant or mixing mode chosen for
+ * FP64 selects the FP64 arithmetic instead).  Variants differ only in the order
+ * of the sums, except 5 (FP16 rounding of the projection), 10 (products of the
+ * TF32 terms) and the FP64 default (its own rounding, below FP64's).  Numbers 1, 2, 6 and 8 are not used.
  * Errors: DWF_EINVAL (NULL handle or pointer, bad prec, variant not -1, 0, 3,
  * 4, 5, 7, 9 or 10, ns or sb outside the ranges above, sb making a CTA of more
  * than 256 threads). */

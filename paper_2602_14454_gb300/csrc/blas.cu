@@ -1,7 +1,7 @@
 // Site-local kernels: fifth-direction mixing, CG vector updates, packing
 // between the canonical complex-double layout and the internal layout,
 // precision conversion, norms, index tables and link preparation.
-#include "fields.cuh"
+#include "fx_fields.cuh"
 
 namespace dwf {
 namespace {
@@ -264,6 +264,14 @@ __global__ void pack_full_kernel(const double *canon, FieldRef even, FieldRef od
         double2 v[12];
         if (!unpack) {
             canon_to_pairs(c, v);
+            if constexpr (P == DWF_F64) {
+                if (f.fx) {   // as blocks
+                    longlong2 t[12];
+                    const int e = fx_pack(v, FX_BITS, t);
+                    fx_st(f, (size_t)site, s, Ls, t, e);
+                    continue;
+                }
+            }
             st_pairs<P>(f, (size_t)site, s, Ls, v);
         } else {
             ld_pairs<P, false>(f, (size_t)site, s, Ls, v);
@@ -493,7 +501,7 @@ cudaError_t launch_mix(int prec, const MixArgs &a, cudaStream_t st)
 cudaError_t launch_cg_update(int prec, const CgUpdateArgs &a, cudaStream_t st)
 {
     switch (prec) {
-    case DWF_F64: return launch_cg_update_t<DWF_F64>(a, st);
+    case DWF_F64: return a.mat_fx ? launch_cg_update_fx(a, st) : launch_cg_update_t<DWF_F64>(a, st);
     case DWF_F32: return launch_cg_update_t<DWF_F32>(a, st);
     case DWF_F16: return launch_cg_update_t<DWF_F16>(a, st);
     }

@@ -5,6 +5,7 @@
 #include <string>
 
 #include "dwf_internal.h"
+#include "fixed.cuh"
 
 using namespace dwf;
 
@@ -109,10 +110,18 @@ FieldRef dwf_ctx::field(const std::string &name, int prec, cudaError_t *err)
     const size_t fb = field_bytes(prec, Vh + ghost, Ls);   // a slab's fields carry its ghost faces
     const size_t sb = scale_bytes(prec, Vh + ghost, Ls);
     const size_t off = (fb + 255) & ~(size_t)255;
-    char *p = (char *)ws(name + "#" + std::to_string(prec), off + sb, err);
+    // an FP64 field has room for the exponents of its block form (blocks() below)
+    const size_t xb = prec == DWF_F64 ? exponent_bytes(Vh + ghost, Ls) : 0;
+    char *p = (char *)ws(name + "#" + std::to_string(prec), off + sb + xb, err);
     if (!p) return f;
     f.v = p;
     f.scale = sb ? (float *)(p + off) : nullptr;
+    return f;
+}
+
+FieldRef dwf_ctx::blocks(FieldRef f) const
+{
+    f.fx = (int *)((char *)f.v + ((field_bytes(DWF_F64, Vh + ghost, Ls) + 255) & ~(size_t)255));
     return f;
 }
 
@@ -193,8 +202,43 @@ HopArgs with_programs_mode(dwf_ctx *h, int prec, const HopArgs &a0, int mode)
 
 HopArgs with_programs(dwf_ctx *h, int prec, const HopArgs &a0) { return with_programs_mode(h, prec, a0, -1); }
 
+// The FP64 launches below run on fixed-point blocks unless the caller chose an FP64
+// hop variant or mixing mode (dwf_ctx::use_fx); block fields reach the others only
+// through a call site that asks use_fx() itself.
+static cudaError_t hop_fx(dwf_ctx *h, bool dag, const HopArgs &a0, cudaStream_t st)
+{
+    HopArgs a = a0;
+    const int ip = mat_id_of(h, DWF_F64, a.post), iy = mat_id_of(h, DWF_F64, a.ymat), iz = mat_id_of(h, DWF_F64, a.zmat);
+    if (ip < 0 || (a.ymat && iy < 0) || (a.zmat && iz < 0)) return cudaErrorInvalidValue;
+    a.post_fx = h->mat_fx(ip);
+    a.post_band = h->band_fx(ip);
+    if (iy >= 0) a.y_fx = h->mat_fx(iy), a.y_band = h->band_fx(iy);
+    if (iz >= 0) a.z_fx = h->mat_fx(iz), a.z_band = h->band_fx(iz);
+    if (!a.in.fx) {   // an FP64 input (a caller that keeps FP64 fields): its blocks first
+        cudaError_t e = cudaSuccess;
+        FieldRef t = h->field("fx_in", DWF_F64, &e);
+        if (!t.v) return e;
+        t = h->blocks(t);
+        h->launches += 1;
+        if ((e = launch_to_blocks(a.in, t, h->Vh + h->ghost, h->Ls, st)) != cudaSuccess) return e;
+        a.in = t;
+    }
+    h->launches += 1;
+    return launch_hop_fx(dag, a, st);
+}
+
+// The hop in FP64 arithmetic whatever the default: the 5D source, whose coefficients
+// are often exact (c = 0 copies b4), has to come out as exact as FP64 makes it.
+cudaError_t hop_fp64(dwf_ctx *h, const HopArgs &a, cudaStream_t st)
+{
+    h->launches += 1;
+    return launch_hop(DWF_F64, false, with_programs(h, DWF_F64, a), h->hop_var[DWF_F64], h->hop_ns[DWF_F64],
+                      h->hop_sb[DWF_F64], st);
+}
+
 cudaError_t hop(dwf_ctx *h, int prec, bool dag, const HopArgs &a, cudaStream_t st)
 {
+    if (prec == DWF_F64 && h->use_fx()) return hop_fx(h, dag, a, st);
     h->launches += 1;
     return launch_hop(prec, dag, with_programs(h, prec, a), h->hop_var[prec], h->hop_ns[prec], h->hop_sb[prec], st);
 }
@@ -213,6 +257,12 @@ cudaError_t hop_cg_plain(dwf_ctx *h, int prec, bool dag, const HopArgs &a, cudaS
     return launch_hop(prec, dag, with_programs_mode(h, prec, a, 1), 9, h->hop_ns[prec], h->hop_sb[prec], st);
 }
 
+// A field that only hops and mixings read: FP64 fields are kept as blocks then.
+FieldRef hop_input(const dwf_ctx *h, int prec, FieldRef f)
+{
+    return prec == DWF_F64 && h->use_fx() ? h->blocks(f) : f;
+}
+
 cudaError_t mix(dwf_ctx *h, int prec, FieldRef in, FieldRef out, int id, cudaStream_t st)
 {
     MixArgs m;
@@ -226,6 +276,11 @@ cudaError_t mix(dwf_ctx *h, int prec, FieldRef in, FieldRef out, int id, cudaStr
     m.band = h->fm.band[id];
     m.err = h->errflag();
     h->launches += 1;
+    if (prec == DWF_F64 && h->use_fx()) {
+        m.mat_fx = h->mat_fx(id);
+        m.band = h->band_fx(id);
+        return launch_mix_fx(m, st);
+    }
     return launch_mix(prec, m, st);
 }
 
@@ -361,6 +416,20 @@ static int create_impl(const int dims[4], int Ls, double M0, double mf, const do
     if ((e = cudaMemcpy(h->mats_dev[1], mf32.data(), mf32.size() * 4, cudaMemcpyHostToDevice)) != cudaSuccess)
         return fail(e, "cudaMemcpy");
     {
+        // fixed-point constants: value = mantissa 2^(exponent - B), below 2^B in magnitude
+        const int B = fx_mix_bits(Ls);
+        std::vector<int4> mx(per * MAT_COUNT);
+        for (size_t k = 0; k < mx.size(); ++k) {
+            int ex = FX_ZERO;
+            const double f = md[k] != 0.0 ? std::frexp(md[k], &ex) : 0.0;
+            const long long m = (long long)std::ldexp(f, B);
+            mx[k] = make_int4((int)(unsigned)m, (int)(m >> 32), ex, 0);
+        }
+        if ((e = cudaMalloc(&h->mats_fx, mx.size() * sizeof(int4))) != cudaSuccess) return fail(e, "cudaMalloc");
+        if ((e = cudaMemcpy(h->mats_fx, mx.data(), mx.size() * sizeof(int4), cudaMemcpyHostToDevice)) != cudaSuccess)
+            return fail(e, "cudaMemcpy");
+    }
+    {
         // structured programs, FP64 and FP32 copies
         std::vector<MixProg<double>> pd(MAT_COUNT);
         std::vector<MixProg<float>> pf(MAT_COUNT);
@@ -424,7 +493,7 @@ static int create_impl(const int dims[4], int Ls, double M0, double mf, const do
     }
     if ((e = launch_build_tables(h->dims, h->nbr, h->eo2lex, 0)) != cudaSuccess) return fail(e, "build_tables");
     if ((e = cudaDeviceSynchronize()) != cudaSuccess) return fail(e, "build_tables");
-    h->bytes = md.size() * 8 + mf32.size() * 4 + (size_t)2 * h->Vh * 9 * sizeof(int) + ((size_t)h->Vh + 8192) * 8;
+    h->bytes = md.size() * (8 + sizeof(int4)) + mf32.size() * 4 + (size_t)2 * h->Vh * 9 * sizeof(int) + ((size_t)h->Vh + 8192) * 8;
     *out = h;
     return DWF_OK;
 }
@@ -440,6 +509,7 @@ int dwf_destroy(dwf_handle h)
         if (h->mats_dev[k]) cudaFree(h->mats_dev[k]);
         if (h->gauge[k]) cudaFree(h->gauge[k]);
     }
+    if (h->mats_fx) cudaFree(h->mats_fx);
     for (int k = 0; k < 2; ++k)
         if (h->progs_dev[k]) cudaFree(h->progs_dev[k]);
     if (h->nbr) cudaFree(h->nbr);
@@ -522,8 +592,10 @@ static int apply_impl(dwf_handle h, int op, int prec, const void *in, void *out,
         FieldRef ye = h->field("ap_ye", prec, &e), yo = h->field("ap_yo", prec, &e);
         FieldRef he = h->field("ap_he", prec, &e), ho = h->field("ap_ho", prec, &e);
         if (!xe.v || !xo.v || !ye.v || !yo.v || !he.v || !ho.v) return dwf_cuda_error(e, "workspace");
+        xe = hop_input(h, prec, xe), xo = hop_input(h, prec, xo);
         CK(launch_pack_full(prec, (const double *)in, xe, xo, h->eo2lex, h->Vh, h->V, h->Ls, st));
         h->launches += 2;   // pack + unpack below
+        he = hop_input(h, prec, he), ho = hop_input(h, prec, ho);
         if (!dag) {
             CK(mix(h, prec, xe, he, MAT_P, st));
             CK(mix(h, prec, xo, ho, MAT_P, st));
@@ -552,6 +624,7 @@ static int apply_impl(dwf_handle h, int op, int prec, const void *in, void *out,
         if (!x.v || !xh.v || !t.v || !y.v) return dwf_cuda_error(e, "workspace");
         CK(launch_pack_eo(prec, (const double *)in, x, h->Vh, h->Ls, st));
         h->launches += 2;   // pack + unpack below
+        xh = hop_input(h, prec, xh), t = hop_input(h, prec, t);
         CK(mix(h, prec, x, xh, dag ? MAT_QT : MAT_P, st));
         HopArgs a1 = hop_args(h, prec, 1, xh, t, dag ? MAT_MT : MAT_M);
         CK(hop(h, prec, dag, a1, st));
@@ -880,7 +953,7 @@ int dwf_source_5d(dwf_handle h, const void *b4, void *b5, void *stream)
         a.y = par ? vo : ve;
         a.ymode = 2;
         a.ymat = h->mat(DWF_F64, MAT_SRC_Y);
-        CK(hop(h, DWF_F64, false, a, st));
+        CK(hop_fp64(h, a, st));
     }
     CK(launch_unpack_full(DWF_F64, oe, oo, (double *)b5, h->eo2lex, h->Vh, h->V, h->Ls, st));
     return DWF_OK;
@@ -1058,7 +1131,7 @@ int dwf_autotune(dwf_handle h, int prec, const char *cache_path, void *stream)
                     h->hop_ns[prec] = ns;
                     h->hop_sb[prec] = sb;
                     h->mixmode[prec] = mix;
-                    h->mixmode[prec] = h->mix_mode(prec);
+                    if (mix >= 0) h->mixmode[prec] = h->mix_mode(prec);
                     hit = true;
                 }
             }
@@ -1068,6 +1141,13 @@ int dwf_autotune(dwf_handle h, int prec, const char *cache_path, void *stream)
     }
     double best = 1e30;
     int bvar = -1, bns = 0, bsb = 0, bmix = 0;
+    if (prec == DWF_F64) {   // the fixed-point hop, the default, has no variant number or mixing mode of its own
+        h->mixmode[prec] = h->hop_var[prec] = bmix = -1;
+        h->hop_ns[prec] = h->hop_sb[prec] = 0;
+        double by = 0;
+        int rc = dwf_time_hop(h, prec, 10, 0, &best, &by, stream);
+        if (rc) return rc;
+    }
     for (int mix = 0; mix <= 2; ++mix)
         for (int var = 0; var <= 10; ++var)
             for (int ns = 1; ns <= 4; ns *= 2) {
@@ -1179,6 +1259,11 @@ int dwf_time_hop(dwf_handle h, int prec, int reps, int flush_l2, double *us, dou
     if (flush_l2) {
         flush = h->ws("th_flush", flush_bytes, &e);
         if (!flush) return dwf_cuda_error(e, "workspace");
+    }
+    if (prec == DWF_F64 && h->use_fx()) {   // blocks of exponent 0
+        in = hop_input(h, prec, in), out = hop_input(h, prec, out);
+        CK(cudaMemsetAsync(in.v, 0x03, field_bytes(prec, h->Vh, h->Ls), st));
+        CK(cudaMemsetAsync(in.fx, 0, exponent_bytes(h->Vh, h->Ls), st));
     }
     HopArgs a = hop_args(h, prec, 1, in, out, MAT_M);
     cudaEvent_t e0, e1;

@@ -74,10 +74,13 @@ struct CgScalars {
 
 enum RedOp { RED_NONE = 0, RED_STORE = 1, RED_CG_ALPHA = 2, RED_CG_BETA = 3, RED_GAMMA = 4 };
 
-// A field in internal layout; scale is non-null for FP16 fields only.
+// A field in internal layout; scale is non-null for FP16 fields only.  fx
+// non-null: an FP64 field held as fixed-point blocks (fixed.cuh), one exponent
+// per (site, s), [site][Ls].
 struct FieldRef {
     void *v = nullptr;
     float *scale = nullptr;
+    int *fx = nullptr;
 };
 
 struct RedArgs {
@@ -115,6 +118,8 @@ struct HopArgs {
     const void *post_prog = nullptr, *y_prog = nullptr, *z_prog = nullptr;
     const int *skip = nullptr;     // batched launches: the system is left untouched while *skip != 0
     int post_band = 0, y_band = 0, z_band = 0;   // the matrix is cyclic tridiagonal (dense mode reads 3 per row)
+    // fixed-point FP64 hop: the matrices' constants (mats_fx), with *_band 2 for a diagonal matrix
+    const int4 *post_fx = nullptr, *y_fx = nullptr, *z_fx = nullptr;
     int zblock = 0;                // sweep the lattice in columns of zblock z-planes (0: index order)
 };
 
@@ -126,6 +131,7 @@ struct MixArgs {
     const void *prog = nullptr;
     int band = 0;
     int *err = nullptr;            // bit 0 set when a bounded device wait gave up (tensor-core form)
+    const int4 *mat_fx = nullptr;  // fixed-point FP64 mixing
 };
 
 // p = r + beta p ; phat = P p   (or with init: p = r)
@@ -139,6 +145,7 @@ struct CgUpdateArgs {
     const void *prog = nullptr;
     const int *skip = nullptr;     // batched launches: the system is left untouched while *skip != 0
     int band = 0;
+    const int4 *mat_fx = nullptr;  // fixed-point FP64 mixing: phat is a block field
     // if set, xacc += scal->alpha * p (p before its update): the x update of the
     // previous CG iteration, deferred to this launch, which reads p anyway
     // (FP64 accumulator for FP64 fields, else FP32)
@@ -171,6 +178,12 @@ int hop_default_variant(int prec);
 int hop_default_ns(int prec, int Ls);
 int hop_default_sb(int prec, int Ls, int ns);
 cudaError_t launch_mix(int prec, const MixArgs &a, cudaStream_t st);
+// Fixed-point FP64 (hop_fx.cuh, mix_fx.cu): the hop from a block field, the mixing
+// and the CG update into one, and FP64 fields of `rows` sites to blocks.
+cudaError_t launch_hop_fx(bool dag, const HopArgs &a, cudaStream_t st);
+cudaError_t launch_mix_fx(const MixArgs &a, cudaStream_t st);
+cudaError_t launch_cg_update_fx(const CgUpdateArgs &a, cudaStream_t st);
+cudaError_t launch_to_blocks(FieldRef in, FieldRef out, int rows, int Ls, cudaStream_t st);
 // the same on the tensor cores (tcgen05, TMEM; FP32 and FP16 fields, Ls <= 32)
 cudaError_t launch_mix_tc(int prec, const MixArgs &a, cudaStream_t st);
 cudaError_t launch_cg_update(int prec, const CgUpdateArgs &a, cudaStream_t st);
@@ -214,6 +227,8 @@ cudaError_t launch_chiral_embed(const double *b4, double *b5, int V, int Ls, cud
 // bytes of one internal half field
 size_t field_bytes(int prec, int Vh, int Ls);
 size_t scale_bytes(int prec, int Vh, int Ls);
+// bytes of the exponents of an FP64 field held as blocks, at the next multiple of 256 behind it
+size_t exponent_bytes(int Vh, int Ls);
 
 // ------------------------------------------------------------ host side
 struct FifthMatrices {
@@ -225,6 +240,7 @@ struct FifthMatrices {
     // nonzeros only on the cyclic tridiagonal (t = s - 1, s, s + 1): the dense
     // mixing then reads three coefficients per row (P, P^T, A5 R, diagonals)
     bool band[MAT_COUNT] = {};
+    bool diag[MAT_COUNT] = {};   // nonzeros only on the diagonal (implies band)
     // structured form of every matrix (see MixProg); valid when `structured`
     bool structured = false;
     struct Prog {
@@ -274,6 +290,12 @@ struct dwf_ctx {
     int device;
     dwf::FifthMatrices fm;
     void *mats_dev[3] = {nullptr, nullptr, nullptr};   // double / float / float copies (F16 uses float)
+    void *mats_fx = nullptr;                           // int4 [MAT_COUNT][2][Ls][Ls]: fixed-point constants
+    const int4 *mat_fx(int id) const { return (const int4 *)mats_fx + (size_t)2 * Ls * Ls * id; }
+    int band_fx(int id) const { return fm.diag[id] ? 2 : (fm.band[id] ? 1 : 0); }
+    // the FP64 operator runs on fixed-point blocks unless the caller chose an FP64 hop
+    // variant or mixing mode of its own
+    bool use_fx() const { return hop_var[DWF_F64] < 0 && mixmode[DWF_F64] < 0; }
     void *progs_dev[2] = {nullptr, nullptr};           // MixProg<double>[MAT_COUNT], MixProg<float>[MAT_COUNT]
     int mixmode[3] = {-1, -1, -1};    // fifth-direction mixing per precision: 0 dense, 1 structured, 2 tensor cores, -1 default
     int mix_mode(int prec) const;
@@ -311,6 +333,8 @@ struct dwf_ctx {
     // named workspace buffer (allocated on first use, grown if needed)
     void *ws(const std::string &name, size_t bytes_needed, cudaError_t *err);
     dwf::FieldRef field(const std::string &name, int prec, cudaError_t *err);
+    // the same FP64 field seen as a block field (its exponents lie behind it)
+    dwf::FieldRef blocks(dwf::FieldRef f) const;
 };
 
 namespace dwf {

@@ -1,0 +1,308 @@
+// Device helpers of the fixed-point FP64 kernels: blocks in memory, the mixing
+// tile, fifth-direction mixing and the epilogue's conversions (arithmetic in
+// fixed.cuh, field layout in dwf_internal.h).
+//
+// A block field stores the field's 16-byte vectors with 64-bit integers in the
+// place of the doubles, and one exponent per (site, s), [site][Ls] int32, behind
+// it (FieldRef::fx).  Registers hold a block as 12 pairs in the order of the FP64
+// kernels (even pairs P_+, odd pairs P_-), so project() and reconstruct() of
+// stencil.cuh apply to it as they are.
+#pragma once
+
+#include "fields.cuh"
+#include "fixed.cuh"
+
+namespace dwf {
+
+template <> struct PairReal<longlong2> { typedef long long R; };
+__device__ __forceinline__ longlong2 p_make(long long a, long long b) { return make_longlong2(a, b); }
+__device__ __forceinline__ longlong2 p_splat(long long a) { return make_longlong2(a, a); }
+__device__ __forceinline__ longlong2 p_fma(longlong2 a, longlong2 b, longlong2 c)
+{
+    return make_longlong2(a.x * b.x + c.x, a.y * b.y + c.y);
+}
+__device__ __forceinline__ longlong2 p_add(longlong2 a, longlong2 b) { return make_longlong2(a.x + b.x, a.y + b.y); }
+
+namespace {
+
+// ------------------------------------------------------------ blocks in memory
+template <bool RO>
+__device__ __forceinline__ void fx_ld(const FieldRef &f, size_t site, int s, int Ls, longlong2 *v)
+{
+    const longlong2 *p = reinterpret_cast<const longlong2 *>(f.v) + (site * 12) * Ls + s;
+#pragma unroll
+    for (int k = 0; k < 12; ++k) v[k] = RO ? __ldg(p + (size_t)k * Ls) : p[(size_t)k * Ls];
+}
+__device__ __forceinline__ void fx_st(const FieldRef &f, size_t site, int s, int Ls, const longlong2 *v, int e)
+{
+    longlong2 *p = reinterpret_cast<longlong2 *>(f.v) + (site * 12) * Ls + s;
+#pragma unroll
+    for (int k = 0; k < 12; ++k) p[(size_t)k * Ls] = v[k];
+    f.fx[site * Ls + s] = e;
+}
+
+// the exponent (or mark) of 12 pairs of doubles
+__device__ __forceinline__ int fx_block_exponent(const double2 *v)
+{
+    uint32_t m = 0, low = 0;
+#pragma unroll
+    for (int k = 0; k < 12; ++k) {
+        m = max(m, max((uint32_t)__double2hiint(v[k].x) & 0x7fffffffu, (uint32_t)__double2hiint(v[k].y) & 0x7fffffffu));
+        low |= (uint32_t)__double2loint(v[k].x) | (uint32_t)__double2loint(v[k].y);
+    }
+    return fx_exponent(m, low);
+}
+// doubles -> integers of B bits below 2^e; a marked block keeps the doubles' bits
+__device__ __forceinline__ int fx_pack(const double2 *v, int B, longlong2 *t)
+{
+    const int e = fx_block_exponent(v);
+#pragma unroll
+    for (int k = 0; k < 12; ++k)
+        t[k] = e == FX_RAW ? make_longlong2(__double_as_longlong(v[k].x), __double_as_longlong(v[k].y))
+                           : make_longlong2(fx_from_double(v[k].x, e, B), fx_from_double(v[k].y, e, B));
+    return e;
+}
+__device__ __forceinline__ void fx_unpack(const longlong2 *t, int e, int B, double2 *v)
+{
+#pragma unroll
+    for (int k = 0; k < 12; ++k)
+        v[k] = e == FX_RAW ? make_double2(__longlong_as_double(t[k].x), __longlong_as_double(t[k].y))
+                           : make_double2(fx_to_double(t[k].x, e - B), fx_to_double(t[k].y, e - B));
+}
+// v[12] <- an FP64 or block field as doubles
+template <bool RO>
+__device__ __forceinline__ void fx_ld_double(const FieldRef &f, size_t site, int s, int Ls, double2 *v)
+{
+    if (f.fx) {
+        longlong2 t[12];
+        fx_ld<RO>(f, site, s, Ls, t);
+        fx_unpack(t, f.fx[site * Ls + s], FX_BITS, v);
+    } else {
+        ld_pairs<DWF_F64, RO>(f, site, s, Ls, v);
+    }
+}
+
+// bits of the largest of the pairs k = first, first + step, ...
+template <int STEP>
+__device__ __forceinline__ int fx_pairs_width(const longlong2 *v, int first)
+{
+    uint32_t hi = 0, lo = 0;
+#pragma unroll
+    for (int k = 0; k < 12; k += STEP) {
+        const longlong2 q = v[k + first];
+        const int32_t hx = (int32_t)(q.x >> 32), hy = (int32_t)(q.y >> 32);
+        hi |= (uint32_t)(hx ^ (hx >> 31)) | (uint32_t)(hy ^ (hy >> 31));
+        lo |= (uint32_t)((int32_t)q.x ^ (hx >> 31)) | (uint32_t)((int32_t)q.y ^ (hy >> 31));
+    }
+    // a set of zeros and minus ones has no bits above the sign: one, so that fx_align shifts by at most 62
+    const int w = hi ? 64 - __clz((int)hi) : 32 - __clz((int)lo);
+    return w > 0 ? w : 1;
+}
+__device__ __forceinline__ bool fx_all_zero(const longlong2 *v)
+{
+    unsigned long long any = 0;
+#pragma unroll
+    for (int k = 0; k < 12; ++k) any |= (unsigned long long)v[k].x | (unsigned long long)v[k].y;
+    return any == 0;
+}
+
+// ------------------------------------------------------------------ the tile
+// Tile rows of one (site, s): 12 vectors of 16 bytes, each two reals as limbs
+// (low, high; radix 2^29), rows 13 vectors apart so that eight lanes' 16-byte
+// accesses hit distinct banks; te[site row] the exponents.  A marked row holds
+// raw doubles.
+constexpr int FX_ROW = 13;
+__host__ __device__ constexpr int fx_site_stride(int Ls) { return Ls * FX_ROW + 1; }
+
+__device__ __forceinline__ void fx_put(int4 *row, const longlong2 *t, int e)
+{
+#pragma unroll
+    for (int k = 0; k < 12; ++k) {
+        int4 q;
+        if (e == FX_RAW) {
+            q = make_int4((int)t[k].x, (int)(t[k].x >> 32), (int)t[k].y, (int)(t[k].y >> 32));
+        } else {
+            fx_limbs29(t[k].x, q.x, q.y);
+            fx_limbs29(t[k].y, q.z, q.w);
+        }
+        row[k] = q;
+    }
+}
+__device__ __forceinline__ double fx_tile_double(int lo, int hi, int e, int B)
+{
+    return e == FX_RAW ? __hiloint2double(hi, lo) : fx_to_double(((int64_t)hi << 29) + lo, e - B);
+}
+
+// A fifth-direction matrix: constants {mantissa low, high word, exponent, 0} of B
+// bits, [chi][t][s], the same entries as doubles, and its kind.
+struct FxMat {
+    const int4 *c;
+    const double *m;
+    int band;   // 0 dense, 1 cyclic tridiagonal, 2 diagonal
+};
+
+// E[chi] of output s: the largest exponent of M_st x_t over the rows t; also the
+// largest row exponent, for the mark.
+__device__ __forceinline__ int fx_mix_exponents(const FxMat &M, const int *te, int s, int Ls, int *E)
+{
+    const int n = M.band == 0 ? Ls : (M.band == 1 ? 3 : 1);
+    int t = M.band == 1 ? (s ? s - 1 : Ls - 1) : s, mark = FX_ZERO;
+    const int4 *c = M.c + s;
+    E[0] = E[1] = 2 * FX_ZERO;
+#pragma unroll 4
+    for (int i = 0; i < n; ++i) {
+        const int e = te[t];
+        mark = max(mark, e);
+        E[0] = max(E[0], __ldg(&c[t * Ls].z) + e);
+        E[1] = max(E[1], __ldg(&c[(Ls + t) * Ls].z) + e);
+        t = t + 1 < Ls ? t + 1 : 0;
+    }
+    return mark;
+}
+
+// r[k] (pairs of chirality CHI only): (M tile)(s) = r 2^(E + 58 - 2 B).  Every product
+// M_st x_t is taken against E by shifting the constant, so a small row next to large
+// ones loses nothing that FP64 would have kept.  Constants that vanish there are
+// skipped, and those below 2^28 take one multiply-add instead of three: the
+// inverse's entries fall off by a factor kappa per slice (0.023 for b 1.5, c 0.5).
+// Lane s starts at row s, so that a warp meets constants of one size together.
+template <int CHI>
+__device__ __forceinline__ void fx_mix_chi(const FxMat &M, const int4 *tile, const int *te, int s, int Ls, int E,
+                                           longlong2 *r)
+{
+    const int n = M.band == 0 ? Ls : (M.band == 1 ? 3 : 1);
+    int t = M.band == 1 ? (s ? s - 1 : Ls - 1) : s;
+    const int4 *c = M.c + CHI * Ls * Ls + s;
+    int64_t hh[12], x[12];
+#pragma unroll
+    for (int k = 0; k < 12; ++k) hh[k] = 0, x[k] = 1 << 28;   // the cross sums are rounded at 2^29
+#pragma unroll 1
+    for (int i = 0; i < n; ++i) {
+        const int4 q = __ldg(&c[t * Ls]);
+        const int sh = E - (q.z + te[t]);
+        const int4 *row = tile + t * FX_ROW + CHI;
+        t = t + 1 < Ls ? t + 1 : 0;
+        if (sh >= 58) continue;
+        const int64_t m = (((int64_t)q.y << 32) | (uint32_t)q.x) >> sh;
+        if (sh >= 30) {   // the constant, below 2^28, is its low limb
+#pragma unroll
+            for (int k = 0; k < 6; ++k) {
+                const int4 v = row[2 * k];
+                x[2 * k] = fx_mad1(v.y, (int32_t)m, x[2 * k]);
+                x[2 * k + 1] = fx_mad1(v.w, (int32_t)m, x[2 * k + 1]);
+            }
+            continue;
+        }
+        int32_t cl, ch;
+        fx_limbs29(m, cl, ch);
+#pragma unroll
+        for (int k = 0; k < 6; ++k) {
+            const int4 v = row[2 * k];
+            fx_mad(v.x, v.y, cl, ch, hh[2 * k], x[2 * k]);
+            fx_mad(v.z, v.w, cl, ch, hh[2 * k + 1], x[2 * k + 1]);
+        }
+    }
+#pragma unroll
+    for (int k = 0; k < 6; ++k)
+        r[2 * k + CHI] = make_longlong2(hh[2 * k] + (x[2 * k] >> 29), hh[2 * k + 1] + (x[2 * k + 1] >> 29));
+}
+
+// the same product in FP64, for rows with non-finite entries: o = M tile
+__device__ __noinline__ void fx_mix_raw(const FxMat &M, const int4 *tile, const int *te, int s, int Ls, int B, double2 *o)
+{
+    for (int k = 0; k < 12; ++k) o[k] = make_double2(0.0, 0.0);
+    for (int t = 0; t < Ls; ++t) {
+        const int dt = t - s < 0 ? t - s + Ls : t - s;
+        if ((M.band == 1 && dt > 1 && dt < Ls - 1) || (M.band == 2 && dt != 0)) continue;
+        for (int k = 0; k < 12; ++k) {
+            const double m = M.m[(size_t)(k & 1) * Ls * Ls + (size_t)t * Ls + s];
+            if (m == 0.0) continue;   // a row that the matrix does not couple
+            const int4 q = tile[t * FX_ROW + k];
+            o[k].x = fma(m, fx_tile_double(q.x, q.y, te[t], B), o[k].x);
+            o[k].y = fma(m, fx_tile_double(q.z, q.w, te[t], B), o[k].y);
+        }
+    }
+}
+
+// A mixing's result: 12 pairs r of 2^(E[chi] + 58 - 2 B) or, where a row that enters
+// holds non-finite values, the doubles' bits (raw).
+struct FxSum {
+    longlong2 r[12];
+    int E[2];
+    bool raw;
+};
+__device__ __forceinline__ void fx_mix(const FxMat &M, const int4 *tile, const int *te, int s, int Ls, int B, FxSum &S)
+{
+    S.raw = fx_mix_exponents(M, te, s, Ls, S.E) >= FX_RAW;
+    if (S.raw) {
+        double2 o[12];
+        fx_mix_raw(M, tile, te, s, Ls, B, o);
+#pragma unroll
+        for (int k = 0; k < 12; ++k) S.r[k] = make_longlong2(__double_as_longlong(o[k].x), __double_as_longlong(o[k].y));
+        return;
+    }
+    fx_mix_chi<0>(M, tile, te, s, Ls, S.E[0], S.r);
+    fx_mix_chi<1>(M, tile, te, s, Ls, S.E[1], S.r);
+}
+__device__ __forceinline__ double2 fx_sum_double(const FxSum &S, int k, int B)
+{
+    if (S.raw) return make_double2(__longlong_as_double(S.r[k].x), __longlong_as_double(S.r[k].y));
+    const int e = S.E[k & 1] + 58 - 2 * B;
+    return make_double2(fx_to_double(S.r[k].x, e), fx_to_double(S.r[k].y, e));
+}
+// S += T; both below 2^62 in magnitude, and so is the sum
+__device__ __forceinline__ void fx_sum_add(FxSum &S, const FxSum &T, int B)
+{
+    if (S.raw || T.raw) {
+#pragma unroll
+        for (int k = 0; k < 12; ++k) {
+            const double2 q = p_add(fx_sum_double(S, k, B), fx_sum_double(T, k, B));
+            S.r[k] = make_longlong2(__double_as_longlong(q.x), __double_as_longlong(q.y));
+        }
+        S.raw = true;
+        return;
+    }
+#pragma unroll
+    for (int c = 0; c < 2; ++c) {
+        const int E = max(S.E[c], T.E[c]) + 1, a = min(E - S.E[c], 63), b = min(E - T.E[c], 63);
+        S.E[c] = E;
+#pragma unroll
+        for (int k = c; k < 12; k += 2)
+            S.r[k] = make_longlong2((S.r[k].x >> a) + (T.r[k].x >> b), (S.r[k].y >> a) + (T.r[k].y >> b));
+    }
+}
+
+// out(site, s) <- the doubles o, as an FP64 or a block field
+__device__ __forceinline__ void fx_store_double(const FieldRef &out, size_t site, int s, int Ls, const double2 *o)
+{
+    if (out.fx) {
+        longlong2 t[12];
+        const int e = fx_pack(o, FX_BITS, t);
+        fx_st(out, site, s, Ls, t, e);
+    } else {
+        st_pairs<DWF_F64>(out, site, s, Ls, o);
+    }
+}
+// out(site, s) <- S
+__device__ __forceinline__ void fx_store_sum(const FieldRef &out, size_t site, int s, int Ls, FxSum &S, int B)
+{
+    if (!out.fx || S.raw) {
+        double2 o[12];
+#pragma unroll
+        for (int k = 0; k < 12; ++k) o[k] = fx_sum_double(S, k, B);
+        fx_store_double(out, site, s, Ls, o);
+        return;
+    }
+    const int w[2] = {fx_pairs_width<2>(S.r, 0), fx_pairs_width<2>(S.r, 1)};
+    const int top[2] = {w[0] + S.E[0] + 58 - 2 * B, w[1] + S.E[1] + 58 - 2 * B};   // |value| < 2^top
+    const int e = max(top[0], top[1]);
+#pragma unroll
+    for (int k = 0; k < 12; ++k) {
+        const int c = k & 1, down = 63 - FX_BITS + (e - top[c]);
+        S.r[k] = make_longlong2(fx_align(S.r[k].x, w[c], down), fx_align(S.r[k].y, w[c], down));
+    }
+    fx_st(out, site, s, Ls, S.r, fx_all_zero(S.r) ? FX_ZERO : e);
+}
+
+}  // namespace
+}  // namespace dwf

@@ -9,6 +9,14 @@ template <int P, bool DAG>
 cudaError_t hop_launch_pd(const HopArgs &a, int var, int NS, int SB, cudaStream_t st);
 template <int P, bool DAG>
 cudaError_t hop_batch_launch_pd(const HopArgs *tab, int nsys, const HopArgs &a0, int NS, int SB, cudaStream_t st);
+template <bool DAG>
+cudaError_t hop_fx_launch(const HopArgs &a, cudaStream_t st);   // hop_fx_<dir>.cu
+
+cudaError_t launch_hop_fx(bool dag, const HopArgs &a, cudaStream_t st)
+{
+    if (!a.in.fx || a.xacc) return cudaErrorInvalidValue;   // no accumulator in its epilogue
+    return dag ? hop_fx_launch<true>(a, st) : hop_fx_launch<false>(a, st);
+}
 
 // Defaults from the sweeps on GB300 at 16^3x32 and 32^3x64, Ls 16: FP32 the
 // warp-autonomous variant 9 (83.7 / 1446 us per hop against 102.4 / 1519 us for

@@ -230,6 +230,10 @@ bool build_fifth_matrices_s(int Ls, double M0, double mf, const double *bs, cons
                     }
                 }
         out.band[id] = band;
+        bool diagonal = true;
+        for (int chi = 0; chi < 2; ++chi)
+            for (int k = 0; k < n * n; ++k) diagonal = diagonal && (k % (n + 1) == 0 || out.mats[id][chi][k] == 0.0);
+        out.diag[id] = diagonal;
     }
     // the structured programs assume coefficients independent of s
     if (constant)

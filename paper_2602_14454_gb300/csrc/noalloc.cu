@@ -7,7 +7,7 @@
 // allocation would synchronise the device), so this entry point keeps the
 // four work fields in one file-scope device array instead.
 //
-// The array has a fixed size (kScratchBytes) and, like every file-scope
+// The array has a fixed size (kScratchBytes, and room for block exponents) and, like every file-scope
 // device variable, exists on every GPU that loads the library until the
 // process exits.  Its device address is looked up once per device, on the
 // first call made with that device current.  All calls share it and it keeps
@@ -23,6 +23,7 @@ namespace dwf_detail {
 HopArgs hop_args(dwf_ctx *h, int prec, int out_par, FieldRef in, FieldRef out, int post);
 cudaError_t hop(dwf_ctx *h, int prec, bool dag, const HopArgs &a, cudaStream_t st);
 cudaError_t mix(dwf_ctx *h, int prec, FieldRef in, FieldRef out, int id, cudaStream_t st);
+FieldRef hop_input(const dwf_ctx *h, int prec, FieldRef f);
 }  // namespace dwf_detail
 using namespace dwf_detail;
 
@@ -31,7 +32,11 @@ namespace {
 constexpr size_t kScratchBytes = (size_t)64 << 20;   // 64 MiB
 constexpr int kMaxDevices = 64;
 
-__device__ __align__(256) unsigned char g_scratch[kScratchBytes];
+// the exponents of the two FP64 fields that are held as fixed-point blocks (four
+// bytes per 24 reals), behind the four fields
+constexpr size_t kExponentBytes = 2 * (kScratchBytes / 4 / (24 * sizeof(double)) + 1) * sizeof(int);
+
+__device__ __align__(256) unsigned char g_scratch[kScratchBytes + kExponentBytes];
 
 std::mutex g_mutex;
 void *g_scratch_addr[kMaxDevices];
@@ -84,6 +89,10 @@ extern "C" int dwf_apply_eo_noalloc(dwf_handle h, int prec, int dag, const void 
         f[k].scale = sb ? (float *)(p + fb) : nullptr;
     }
     FieldRef x = f[0], xh = f[1], t = f[2], y = f[3];
+    if (hop_input(h, prec, xh).fx) {
+        xh.fx = (int *)((unsigned char *)base + kScratchBytes);
+        t.fx = xh.fx + (size_t)h->Vh * h->Ls;
+    }
     cudaStream_t st = (cudaStream_t)stream;
     if ((e = launch_pack_eo(prec, (const double *)in, x, h->Vh, h->Ls, st)) != cudaSuccess)
         return dwf_cuda_error(e, "pack");

@@ -36,7 +36,9 @@ HopArgs hop_args(dwf_ctx *h, int prec, int out_par, FieldRef in, FieldRef out, i
 HopArgs with_programs(dwf_ctx *h, int prec, const HopArgs &a0);
 cudaError_t hop(dwf_ctx *h, int prec, bool dag, const HopArgs &a, cudaStream_t st);
 cudaError_t hop_cg_plain(dwf_ctx *h, int prec, bool dag, const HopArgs &a, cudaStream_t st);
+cudaError_t hop_fp64(dwf_ctx *h, const HopArgs &a, cudaStream_t st);
 cudaError_t mix(dwf_ctx *h, int prec, FieldRef in, FieldRef out, int id, cudaStream_t st);
+FieldRef hop_input(const dwf_ctx *h, int prec, FieldRef f);
 RedArgs red(dwf_ctx *h, int op, CgScalars *scal);
 }  // namespace dwf_detail
 using namespace dwf_detail;
@@ -64,6 +66,7 @@ __global__ void reliable_fix_kernel(CgScalars *cg, const CgScalars *fresh, int f
 struct Bufs {
     int ps;   // inner precision
     int xp;   // accumulator precision
+    bool fx = false;   // FP64 inner iterations on blocks: ph, t, wh and u are block fields (iteration_args)
     int form = 0;   // 0: CG on D_pc (eq. even-odd_linear_equation), 1: on D' (eq. another_even-odd_linear_equation)
     FieldRef be, bo, bt, x64, r64, t64, h64, xo64;
     FieldRef p, ph, t, wh, u, rs, xs;
@@ -75,6 +78,7 @@ int get_bufs(dwf_ctx *h, int ps, Bufs &B)
     cudaError_t e = cudaSuccess;
     B.ps = ps;
     B.xp = (ps == DWF_F64) ? DWF_F64 : DWF_F32;
+    B.fx = ps == DWF_F64 && h->use_fx();
     B.be = h->field("sv_be", DWF_F64, &e);
     B.bo = h->field("sv_bo", DWF_F64, &e);
     B.bt = h->field("sv_bt", DWF_F64, &e);
@@ -111,8 +115,10 @@ struct IterArgs {
 // D'^dag w = w - 1/4 M^T H^dag M^T H^dag w (the product P Q of the first form's
 // outer mixings is M, and D_ee Q = 1): p^ = M p, K_b without the Q^T mixing,
 // K_d with the identity in place of Q^-T and -1/4 M^T in place of -1/4 P^T.
-IterArgs iteration_args(dwf_ctx *h, const Bufs &B, const RedArgs &ra, const RedArgs &rb)
+IterArgs iteration_args(dwf_ctx *h, const Bufs &B0, const RedArgs &ra, const RedArgs &rb)
 {
+    Bufs B = B0;
+    if (B.fx) B.ph = h->blocks(B.ph), B.t = h->blocks(B.t), B.wh = h->blocks(B.wh), B.u = h->blocks(B.u);
     const int P = B.ps;
     const bool f2 = B.form == 1;
     IterArgs I;
@@ -127,6 +133,7 @@ IterArgs iteration_args(dwf_ctx *h, const Bufs &B, const RedArgs &ra, const RedA
     ue.mixmode = h->mix_mode(P);
     ue.prog = h->prog(P, pre);
     ue.band = h->fm.band[pre];
+    if (B.fx) ue.mat_fx = h->mat_fx(pre), ue.band = h->band_fx(pre);
     ue.scal = B.cg;
     ue.xacc = B.xs.v;   // x += alpha p of the previous iteration
 
@@ -182,10 +189,11 @@ cudaError_t inner_iteration(dwf_ctx *h, const Bufs &B, cudaStream_t st)
 cudaError_t true_residual(dwf_ctx *h, const Bufs &B, cudaStream_t st)
 {
     cudaError_t e;
-    if ((e = mix(h, DWF_F64, B.x64, B.h64, MAT_P, st)) != cudaSuccess) return e;
-    HopArgs a1 = hop_args(h, DWF_F64, 1, B.h64, B.t64, MAT_M);
+    const FieldRef xh = hop_input(h, DWF_F64, B.h64), t = hop_input(h, DWF_F64, B.t64);
+    if ((e = mix(h, DWF_F64, B.x64, xh, MAT_P, st)) != cudaSuccess) return e;
+    HopArgs a1 = hop_args(h, DWF_F64, 1, xh, t, MAT_M);
     if ((e = hop(h, DWF_F64, false, a1, st)) != cudaSuccess) return e;
-    HopArgs a2 = hop_args(h, DWF_F64, 0, B.t64, B.r64, MAT_NQ4);
+    HopArgs a2 = hop_args(h, DWF_F64, 0, t, B.r64, MAT_NQ4);
     a2.y = B.x64;
     a2.ymode = 1;
     a2.rin = B.bt;
@@ -212,11 +220,12 @@ cudaError_t normal_residual(dwf_ctx *h, const Bufs &B, cudaStream_t st)
     cudaError_t e;
     h->launches += 1;
     if ((e = launch_convert(DWF_F64, B.r64, P, B.rs, h->Vh, h->Ls, st)) != cudaSuccess) return e;
-    if ((e = mix(h, P, B.rs, B.ph, B.form == 1 ? MAT_A5R : MAT_QT, st)) != cudaSuccess) return e;
-    HopArgs a1 = hop_args(h, P, 1, B.ph, B.u, MAT_MT);
+    const FieldRef ph = hop_input(h, P, B.ph), u = hop_input(h, P, B.u);
+    if ((e = mix(h, P, B.rs, ph, B.form == 1 ? MAT_A5R : MAT_QT, st)) != cudaSuccess) return e;
+    HopArgs a1 = hop_args(h, P, 1, ph, u, MAT_MT);
     if ((e = hop(h, P, true, a1, st)) != cudaSuccess) return e;
-    HopArgs a2 = hop_args(h, P, 0, B.u, B.rs, B.form == 1 ? MAT_NMT4 : MAT_NPT4);
-    a2.y = B.form == 1 ? B.ph : B.rs;
+    HopArgs a2 = hop_args(h, P, 0, u, B.rs, B.form == 1 ? MAT_NMT4 : MAT_NPT4);
+    a2.y = B.form == 1 ? ph : B.rs;
     a2.ymode = 1;
     a2.red = red(h, RED_STORE, B.n64);
     return hop(h, P, true, a2, st);
@@ -408,9 +417,10 @@ static int solve_impl(dwf_handle h, const void *b5, void *x5, const dwf_solve_pa
         return DWF_OK;
     }
     // b~_e = Q b_e + 1/2 Q H_eo M b_o
-    CK(mix(h, DWF_F64, B.bo, B.t64, MAT_M, st));
     {
-        HopArgs a = hop_args(h, DWF_F64, 0, B.t64, B.bt, MAT_HALF_Q);
+        const FieldRef t = hop_input(h, DWF_F64, B.t64);
+        CK(mix(h, DWF_F64, B.bo, t, MAT_M, st));
+        HopArgs a = hop_args(h, DWF_F64, 0, t, B.bt, MAT_HALF_Q);
         a.y = B.be;
         a.ymode = 2;
         a.ymat = h->mat(DWF_F64, MAT_Q);
@@ -446,8 +456,8 @@ static int solve_impl(dwf_handle h, const void *b5, void *x5, const dwf_solve_pa
     GraphCache &G = X.graph;
     char keybuf[256];
     // the captured kernels depend on the hop configuration and mixing mode too
-    std::snprintf(keybuf, sizeof keybuf, "%d/%d/%p/%p/%p/%d/%d/%d/%d/%d/%d", ps, N, B.p.v, B.rs.v, B.xs.v,
-                  p->use_graph, h->hop_var[ps], h->hop_ns[ps], h->hop_sb[ps], h->mix_mode(ps), B.form);
+    std::snprintf(keybuf, sizeof keybuf, "%d/%d/%p/%p/%p/%d/%d/%d/%d/%d/%d/%d", ps, N, B.p.v, B.rs.v, B.xs.v,
+                  p->use_graph, h->hop_var[ps], h->hop_ns[ps], h->hop_sb[ps], h->mix_mode(ps), B.form, (int)B.fx);
     if (p->use_graph && G.key != keybuf) {
         if (G.exec) cudaGraphExecDestroy(G.exec);
         G.exec = nullptr;
@@ -595,17 +605,18 @@ static int solve_impl(dwf_handle h, const void *b5, void *x5, const dwf_solve_pa
             }
         }
         // x_o = Q b_o + 1/2 Q H_oe P x_e ; full residual
-        CK(mix(h, DWF_F64, B.x64, B.h64, MAT_P, st));
+        const FieldRef xh = hop_input(h, DWF_F64, B.h64), t = hop_input(h, DWF_F64, B.t64);
+        CK(mix(h, DWF_F64, B.x64, xh, MAT_P, st));
         {
-            HopArgs a = hop_args(h, DWF_F64, 1, B.h64, B.xo64, MAT_HALF_Q);
+            HopArgs a = hop_args(h, DWF_F64, 1, xh, B.xo64, MAT_HALF_Q);
             a.y = B.bo;
             a.ymode = 2;
             a.ymat = h->mat(DWF_F64, MAT_Q);
             CK(hop(h, DWF_F64, false, a, st));
         }
-        CK(mix(h, DWF_F64, B.xo64, B.t64, MAT_P, st));
+        CK(mix(h, DWF_F64, B.xo64, t, MAT_P, st));
         for (int par = 0; par < 2; ++par) {
-            HopArgs a = hop_args(h, DWF_F64, par, par ? B.h64 : B.t64, B.r64, MAT_NHALF);
+            HopArgs a = hop_args(h, DWF_F64, par, par ? xh : t, B.r64, MAT_NHALF);
             a.y = par ? B.xo64 : B.x64;
             a.ymode = 2;
             a.ymat = h->mat(DWF_F64, MAT_A5R);
@@ -666,11 +677,16 @@ struct Arena {
         FieldRef f;
         f.v = take(field_bytes(prec, Vh, Ls));
         if (prec == DWF_F16) f.scale = (float *)take(scale_bytes(prec, Vh, Ls));
+        if (prec == DWF_F64 && f.v && !take(exponent_bytes(Vh, Ls))) f.v = nullptr;   // behind it (dwf_ctx::blocks)
         return f;
     }
 };
 
-size_t field_total(int prec, int Vh, int Ls) { return round256(field_bytes(prec, Vh, Ls)) + round256(scale_bytes(prec, Vh, Ls)); }
+size_t field_total(int prec, int Vh, int Ls)
+{
+    return round256(field_bytes(prec, Vh, Ls)) + round256(scale_bytes(prec, Vh, Ls)) +
+           (prec == DWF_F64 ? round256(exponent_bytes(Vh, Ls)) : 0);
+}
 
 size_t system_bytes(const dwf_ctx *h, int ps)
 {
@@ -709,7 +725,7 @@ cudaError_t source_eo(dwf_ctx *h, const void *b4, double *v5, FieldRef ve, Field
         a.y = par ? vo : ve;
         a.ymode = 2;
         a.ymat = h->mat(DWF_F64, MAT_SRC_Y);
-        if ((e = hop(h, DWF_F64, false, a, st)) != cudaSuccess) return e;
+        if ((e = hop_fp64(h, a, st)) != cudaSuccess) return e;
     }
     return cudaSuccess;
 }
@@ -776,9 +792,10 @@ int sys_prepare(SysRun &R, const void *b4, double *v5, const dwf_solve_params *p
         R.done = true;
         return DWF_OK;
     }
-    CK(mix(h, DWF_F64, B.bo, B.t64, MAT_M, st));
     {
-        HopArgs a = hop_args(h, DWF_F64, 0, B.t64, B.bt, MAT_HALF_Q);
+        const FieldRef t = hop_input(h, DWF_F64, B.t64);
+        CK(mix(h, DWF_F64, B.bo, t, MAT_M, st));
+        HopArgs a = hop_args(h, DWF_F64, 0, t, B.bt, MAT_HALF_Q);
         a.y = B.be;
         a.ymode = 2;
         a.ymat = h->mat(DWF_F64, MAT_Q);
@@ -804,17 +821,18 @@ int sys_finish(SysRun &R, const void *b4, void *x4, double *v5, const dwf_solve_
     dwf_ctx *h = R.h;
     Bufs &B = R.B;
     CK(source_eo(h, b4, v5, B.r64, B.t64, B.be, B.bo, st));
-    CK(mix(h, DWF_F64, B.x64, B.h64, MAT_P, st));
+    const FieldRef xh = hop_input(h, DWF_F64, B.h64), t = hop_input(h, DWF_F64, B.t64);
+    CK(mix(h, DWF_F64, B.x64, xh, MAT_P, st));
     {
-        HopArgs a = hop_args(h, DWF_F64, 1, B.h64, B.xo64, MAT_HALF_Q);
+        HopArgs a = hop_args(h, DWF_F64, 1, xh, B.xo64, MAT_HALF_Q);
         a.y = B.bo;
         a.ymode = 2;
         a.ymat = h->mat(DWF_F64, MAT_Q);
         CK(hop(h, DWF_F64, false, a, st));
     }
-    CK(mix(h, DWF_F64, B.xo64, B.t64, MAT_P, st));
+    CK(mix(h, DWF_F64, B.xo64, t, MAT_P, st));
     for (int par = 0; par < 2; ++par) {
-        HopArgs a = hop_args(h, DWF_F64, par, par ? B.h64 : B.t64, B.r64, MAT_NHALF);
+        HopArgs a = hop_args(h, DWF_F64, par, par ? xh : t, B.r64, MAT_NHALF);
         a.y = par ? B.xo64 : B.x64;
         a.ymode = 2;
         a.ymat = h->mat(DWF_F64, MAT_A5R);

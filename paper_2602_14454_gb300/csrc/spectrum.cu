@@ -18,6 +18,7 @@ namespace dwf_detail {
 HopArgs hop_args(dwf_ctx *h, int prec, int out_par, FieldRef in, FieldRef out, int post);
 cudaError_t hop(dwf_ctx *h, int prec, bool dag, const HopArgs &a, cudaStream_t st);
 cudaError_t mix(dwf_ctx *h, int prec, FieldRef in, FieldRef out, int id, cudaStream_t st);
+FieldRef hop_input(const dwf_ctx *h, int prec, FieldRef f);
 RedArgs red(dwf_ctx *h, int op, CgScalars *scal);
 }  // namespace dwf_detail
 using namespace dwf_detail;
@@ -90,6 +91,7 @@ int normal_apply_f64(dwf_ctx *h, FieldRef x, FieldRef out, cudaStream_t st)
     FieldRef ph = h->field("lz_ph", P, &e), t = h->field("lz_t", P, &e);
     FieldRef wh = h->field("lz_wh", P, &e), u = h->field("lz_u", P, &e);
     if (!ph.v || !t.v || !wh.v || !u.v) return dwf_cuda_error(e, "workspace");
+    ph = hop_input(h, P, ph), t = hop_input(h, P, t), wh = hop_input(h, P, wh), u = hop_input(h, P, u);
     CK(mix(h, P, x, ph, MAT_P, st));
     HopArgs a1 = hop_args(h, P, 1, ph, t, MAT_M);
     CK(hop(h, P, false, a1, st));
@@ -115,6 +117,7 @@ int eo_apply_f64(dwf_ctx *h, FieldRef x, FieldRef out, cudaStream_t st)
     cudaError_t e = cudaSuccess;
     FieldRef ph = h->field("lz_ph", P, &e), t = h->field("lz_t", P, &e);
     if (!ph.v || !t.v) return dwf_cuda_error(e, "workspace");
+    ph = hop_input(h, P, ph), t = hop_input(h, P, t);
     CK(mix(h, P, x, ph, MAT_P, st));
     HopArgs a1 = hop_args(h, P, 1, ph, t, MAT_M);
     CK(hop(h, P, false, a1, st));
@@ -132,6 +135,7 @@ int eo_dag_apply_f64(dwf_ctx *h, FieldRef x, FieldRef out, cudaStream_t st)
     cudaError_t e = cudaSuccess;
     FieldRef wh = h->field("lz_wh", P, &e), u = h->field("lz_u", P, &e);
     if (!wh.v || !u.v) return dwf_cuda_error(e, "workspace");
+    wh = hop_input(h, P, wh), u = hop_input(h, P, u);
     CK(mix(h, P, x, wh, MAT_QT, st));
     HopArgs a1 = hop_args(h, P, 1, wh, u, MAT_MT);
     CK(hop(h, P, true, a1, st));
