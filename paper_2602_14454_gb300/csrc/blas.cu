@@ -1,7 +1,6 @@
-// Site-local kernels: fifth-direction mixing, CG vector updates, packing
-// between the canonical complex-double layout and the internal layout,
-// precision conversion, norms, index tables and link preparation.
-#include "fx_fields.cuh"
+// Site-local kernels: fifth-direction mixing, CG vector updates, precision
+// conversion, norms and index tables.
+#include "fields.cuh"
 
 namespace dwf {
 namespace {
@@ -220,86 +219,6 @@ cudaError_t launch_cg_update_batch_t(const CgUpdateArgs *tab, int nsys, const Cg
                                                          : launch_cg_update_batch_m<P, 0>(tab, nsys, a0, st);
 }
 
-// ------------------------------------------------------------------ packing
-// canonical 24 reals (spin*3 + a)*2 + c  <->  internal pairs (4g + spin, g = 2a + c)
-__device__ __forceinline__ void canon_to_pairs(const double *c, double2 *v)
-{
-    double r[24];
-#pragma unroll
-    for (int k = 0; k < 24; k += 2) {
-        const double2 q = *reinterpret_cast<const double2 *>(c + k);
-        r[k] = q.x;
-        r[k + 1] = q.y;
-    }
-#pragma unroll
-    for (int p = 0; p < 12; ++p)
-        v[p] = make_double2(r[canon_of_internal(2 * p)], r[canon_of_internal(2 * p + 1)]);
-}
-__device__ __forceinline__ void pairs_to_canon(const double2 *v, double *c)
-{
-    double r[24];
-#pragma unroll
-    for (int p = 0; p < 12; ++p) {
-        r[canon_of_internal(2 * p)] = v[p].x;
-        r[canon_of_internal(2 * p + 1)] = v[p].y;
-    }
-#pragma unroll
-    for (int k = 0; k < 24; k += 2) *reinterpret_cast<double2 *>(c + k) = make_double2(r[k], r[k + 1]);
-}
-
-// thread per (parity, eo site, s); canonical full field [s][lex][24 reals]
-template <int P>
-__global__ void pack_full_kernel(const double *canon, FieldRef even, FieldRef odd, const int *eo2lex, int Vh,
-                                 int V, int Ls, int unpack)
-{
-    const size_t n = (size_t)2 * Vh * Ls;
-    for (size_t idx = blockIdx.x * (size_t)blockDim.x + threadIdx.x; idx < n; idx += (size_t)gridDim.x * blockDim.x) {
-        const int s = (int)(idx % Ls);
-        const size_t rest = idx / Ls;
-        const int site = (int)(rest % Vh);
-        const int par = (int)(rest / Vh);
-        const int lex = eo2lex[(size_t)par * Vh + site];
-        const FieldRef &f = par ? odd : even;
-        double *c = const_cast<double *>(canon) + ((size_t)s * V + lex) * 24;
-        double2 v[12];
-        if (!unpack) {
-            canon_to_pairs(c, v);
-            if constexpr (P == DWF_F64) {
-                if (f.fx) {   // as blocks
-                    longlong2 t[12];
-                    const int e = fx_pack(v, FX_BITS, t);
-                    fx_st(f, (size_t)site, s, Ls, t, e);
-                    continue;
-                }
-            }
-            st_pairs<P>(f, (size_t)site, s, Ls, v);
-        } else {
-            ld_pairs<P, false>(f, (size_t)site, s, Ls, v);
-            pairs_to_canon(v, c);
-        }
-    }
-}
-
-// canonical EO field [s][i][24 reals]
-template <int P>
-__global__ void pack_eo_kernel(const double *canon, FieldRef f, int Vh, int Ls, int unpack)
-{
-    const size_t n = (size_t)Vh * Ls;
-    for (size_t idx = blockIdx.x * (size_t)blockDim.x + threadIdx.x; idx < n; idx += (size_t)gridDim.x * blockDim.x) {
-        const int s = (int)(idx % Ls);
-        const int site = (int)(idx / Ls);
-        double *c = const_cast<double *>(canon) + ((size_t)s * Vh + site) * 24;
-        double2 v[12];
-        if (!unpack) {
-            canon_to_pairs(c, v);
-            st_pairs<P>(f, (size_t)site, s, Ls, v);
-        } else {
-            ld_pairs<P, false>(f, (size_t)site, s, Ls, v);
-            pairs_to_canon(v, c);
-        }
-    }
-}
-
 template <int PI, int PO>
 __global__ void convert_kernel(FieldRef in, FieldRef out, int Vh, int Ls)
 {
@@ -367,7 +286,7 @@ __global__ void __launch_bounds__(256) norm2_kernel(FieldRef f, int Vh, int Ls, 
     grid_reduce(acc, red);
 }
 
-// ------------------------------------------------------------ tables, links
+// ------------------------------------------------------------ tables
 __device__ __forceinline__ void eo_coords(int par, int i, const int *d, int c[4])
 {
     const int hx = d[0] / 2;
@@ -390,7 +309,6 @@ __device__ __forceinline__ int eo_of(const int c[4], const int *d)
 
 struct Dims {
     int d[4];
-    int bc[4];
 };
 
 __global__ void tables_kernel(Dims D, int Vh, int *nbr, int *eo2lex)
@@ -412,42 +330,6 @@ __global__ void tables_kernel(Dims D, int Vh, int *nbr, int *eo2lex)
     }
 }
 
-__global__ void pack_gauge_kernel(const double *U, Dims D, int Vh, int V, double *g64, float *g32, __half *g16)
-{
-    const size_t n = (size_t)2 * Vh * 8;
-    for (size_t idx = blockIdx.x * (size_t)blockDim.x + threadIdx.x; idx < n; idx += (size_t)gridDim.x * blockDim.x) {
-        const int dir = (int)(idx % 8);
-        const int i = (int)((idx / 8) % Vh);
-        const int par = (int)(idx / (8 * (size_t)Vh));
-        int c[4];
-        eo_coords(par, i, D.d, c);
-        const int mu = dir & 3;
-        double u[18];
-        if (dir < 4) {
-            const double ph = (c[mu] == D.d[mu] - 1) ? (double)D.bc[mu] : 1.0;
-            const double *src = U + ((size_t)mu * V + lex_of(c, D.d)) * 18;
-            for (int k = 0; k < 18; ++k) u[k] = ph * src[k];
-        } else {
-            int b[4] = {c[0], c[1], c[2], c[3]};
-            b[mu] = (c[mu] - 1 + D.d[mu]) % D.d[mu];
-            const double ph = (c[mu] == 0) ? (double)D.bc[mu] : 1.0;
-            const double *src = U + ((size_t)mu * V + lex_of(b, D.d)) * 18;
-            // dagger: u[a][b] = conj(U[b][a])
-            for (int a = 0; a < 3; ++a)
-                for (int bb = 0; bb < 3; ++bb) {
-                    u[(a * 3 + bb) * 2] = ph * src[(bb * 3 + a) * 2];
-                    u[(a * 3 + bb) * 2 + 1] = -ph * src[(bb * 3 + a) * 2 + 1];
-                }
-        }
-        const size_t o = idx * 18;
-        for (int k = 0; k < 18; ++k) {
-            g64[o + k] = u[k];
-            g32[o + k] = (float)u[k];
-            g16[o + k] = __double2half(u[k]);
-        }
-    }
-}
-
 // x4 = P_- x5(s=1) + P_+ x5(s=Ls)
 __global__ void project4d_kernel(const double *x5, double *x4, int V, int Ls)
 {
@@ -458,22 +340,6 @@ __global__ void project4d_kernel(const double *x5, double *x4, int V, int Ls)
         const int spin = k / 6;
         const int s = (spin < 2) ? (Ls - 1) : 0;
         x4[idx] = x5[((size_t)s * V + site) * 24 + k];
-    }
-}
-
-// v5 = P^dag (0, ..., 0, b4): v(s=1) = P_+ b4, v(s=Ls) = P_- b4, zero elsewhere
-__global__ void chiral_embed_kernel(const double *b4, double *v5, int V, int Ls)
-{
-    const size_t n = (size_t)Ls * V * 24;
-    for (size_t idx = blockIdx.x * (size_t)blockDim.x + threadIdx.x; idx < n; idx += (size_t)gridDim.x * blockDim.x) {
-        const int k = (int)(idx % 24);
-        const size_t site = (idx / 24) % V;
-        const int s = (int)(idx / (24 * (size_t)V));
-        const int spin = k / 6;
-        double v = 0.0;
-        if (s == 0 && spin < 2) v = b4[site * 24 + k];
-        if (s == Ls - 1 && spin >= 2) v = b4[site * 24 + k];
-        v5[idx] = v;
     }
 }
 
@@ -518,56 +384,6 @@ cudaError_t launch_cg_update_batch(int prec, const CgUpdateArgs *tab, int nsys, 
     case DWF_F16: return launch_cg_update_batch_t<DWF_F16>(tab, nsys, a0, st);
     }
     return cudaErrorInvalidValue;
-}
-
-cudaError_t launch_pack_full(int prec, const double *canon, FieldRef even, FieldRef odd, const int *eo2lex, int Vh,
-                             int V, int Ls, cudaStream_t st)
-{
-    const int g = grid_cap((size_t)2 * Vh * Ls);
-    switch (prec) {
-    case DWF_F64: pack_full_kernel<DWF_F64><<<g, kThreads, 0, st>>>(canon, even, odd, eo2lex, Vh, V, Ls, 0); break;
-    case DWF_F32: pack_full_kernel<DWF_F32><<<g, kThreads, 0, st>>>(canon, even, odd, eo2lex, Vh, V, Ls, 0); break;
-    case DWF_F16: pack_full_kernel<DWF_F16><<<g, kThreads, 0, st>>>(canon, even, odd, eo2lex, Vh, V, Ls, 0); break;
-    default: return cudaErrorInvalidValue;
-    }
-    return cudaGetLastError();
-}
-
-cudaError_t launch_unpack_full(int prec, FieldRef even, FieldRef odd, double *canon, const int *eo2lex, int Vh,
-                               int V, int Ls, cudaStream_t st)
-{
-    const int g = grid_cap((size_t)2 * Vh * Ls);
-    switch (prec) {
-    case DWF_F64: pack_full_kernel<DWF_F64><<<g, kThreads, 0, st>>>(canon, even, odd, eo2lex, Vh, V, Ls, 1); break;
-    case DWF_F32: pack_full_kernel<DWF_F32><<<g, kThreads, 0, st>>>(canon, even, odd, eo2lex, Vh, V, Ls, 1); break;
-    case DWF_F16: pack_full_kernel<DWF_F16><<<g, kThreads, 0, st>>>(canon, even, odd, eo2lex, Vh, V, Ls, 1); break;
-    default: return cudaErrorInvalidValue;
-    }
-    return cudaGetLastError();
-}
-
-cudaError_t launch_pack_eo(int prec, const double *canon, FieldRef f, int Vh, int Ls, cudaStream_t st)
-{
-    const int g = grid_cap((size_t)Vh * Ls);
-    switch (prec) {
-    case DWF_F64: pack_eo_kernel<DWF_F64><<<g, kThreads, 0, st>>>(canon, f, Vh, Ls, 0); break;
-    case DWF_F32: pack_eo_kernel<DWF_F32><<<g, kThreads, 0, st>>>(canon, f, Vh, Ls, 0); break;
-    case DWF_F16: pack_eo_kernel<DWF_F16><<<g, kThreads, 0, st>>>(canon, f, Vh, Ls, 0); break;
-    default: return cudaErrorInvalidValue;
-    }
-    return cudaGetLastError();
-}
-
-cudaError_t launch_unpack_eo(int prec, FieldRef f, double *canon, int Vh, int Ls, cudaStream_t st)
-{
-    const int g = grid_cap((size_t)Vh * Ls);
-    switch (prec) {
-    case DWF_F64: pack_eo_kernel<DWF_F64><<<g, kThreads, 0, st>>>(canon, f, Vh, Ls, 1); break;
-    case DWF_F32: pack_eo_kernel<DWF_F32><<<g, kThreads, 0, st>>>(canon, f, Vh, Ls, 1); break;
-    case DWF_F16: pack_eo_kernel<DWF_F16><<<g, kThreads, 0, st>>>(canon, f, Vh, Ls, 1); break;
-    default: return cudaErrorInvalidValue;
-    }
-    return cudaGetLastError();
 }
 
 cudaError_t launch_convert(int pi, FieldRef in, int po, FieldRef out, int Vh, int Ls, cudaStream_t st)
@@ -625,36 +441,16 @@ cudaError_t launch_zero(int prec, FieldRef f, int Vh, int Ls, cudaStream_t st)
 cudaError_t launch_build_tables(const int dims[4], int *nbr, int *eo2lex, cudaStream_t st)
 {
     Dims D;
-    for (int k = 0; k < 4; ++k) D.d[k] = dims[k], D.bc[k] = 1;
+    for (int k = 0; k < 4; ++k) D.d[k] = dims[k];
     const int V = dims[0] * dims[1] * dims[2] * dims[3];
     const int Vh = V / 2;
     tables_kernel<<<grid_cap((size_t)2 * Vh), kThreads, 0, st>>>(D, Vh, nbr, eo2lex);
     return cudaGetLastError();
 }
 
-cudaError_t launch_pack_gauge(const double *U, const int dims[4], const int bc[4], const int *eo2lex, const int *nbr,
-                              void *g64, void *g32, void *g16, cudaStream_t st)
-{
-    (void)eo2lex;
-    (void)nbr;
-    Dims D;
-    for (int k = 0; k < 4; ++k) D.d[k] = dims[k], D.bc[k] = bc[k];
-    const int V = dims[0] * dims[1] * dims[2] * dims[3];
-    const int Vh = V / 2;
-    pack_gauge_kernel<<<grid_cap((size_t)2 * Vh * 8), kThreads, 0, st>>>(
-        U, D, Vh, V, (double *)g64, (float *)g32, (__half *)g16);
-    return cudaGetLastError();
-}
-
 cudaError_t launch_project4d(const double *x5, double *x4, int V, int Ls, cudaStream_t st)
 {
     project4d_kernel<<<grid_cap((size_t)V * 24), kThreads, 0, st>>>(x5, x4, V, Ls);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_chiral_embed(const double *b4, double *b5, int V, int Ls, cudaStream_t st)
-{
-    chiral_embed_kernel<<<grid_cap((size_t)Ls * V * 24), kThreads, 0, st>>>(b4, b5, V, Ls);
     return cudaGetLastError();
 }
 

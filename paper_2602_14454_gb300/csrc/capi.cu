@@ -227,13 +227,48 @@ static cudaError_t hop_fx(dwf_ctx *h, bool dag, const HopArgs &a0, cudaStream_t 
     return launch_hop_fx(dag, a, st);
 }
 
-// The hop in FP64 arithmetic whatever the default: the 5D source, whose coefficients
-// are often exact (c = 0 copies b4), has to come out as exact as FP64 makes it.
-cudaError_t hop_fp64(dwf_ctx *h, const HopArgs &a, cudaStream_t st)
+// h_par = (c / 2) H v over the two walls (slices 1 and Ls of the source), v = P_+- b4
+// in `scratch` (source_scratch_bytes); null fields when c_1 = c_Ls = 0, where the
+// source is b4 itself.  The other slices of the source are zero, so its hop takes
+// two slices of fixed-point blocks, not Ls (24^3x48, Ls 8: 1632 us against 9461 us).
+static size_t half2_bytes(const dwf_ctx *h)
 {
-    h->launches += 1;
-    return launch_hop(DWF_F64, false, with_programs(h, DWF_F64, a), h->hop_var[DWF_F64], h->hop_ns[DWF_F64],
-                      h->hop_sb[DWF_F64], st);
+    const size_t v = (field_bytes(DWF_F64, h->Vh, 2) + 255) & ~(size_t)255;
+    return v + ((exponent_bytes(h->Vh, 2) + 255) & ~(size_t)255);
+}
+size_t source_scratch_bytes(const dwf_ctx *h) { return 4 * half2_bytes(h); }
+
+cudaError_t source_hops(dwf_ctx *h, const void *b4, void *scratch, FieldRef hop2[2], cudaStream_t st)
+{
+    const int n = h->Ls - 1;
+    const std::vector<double> &post = h->fm.mats[MAT_SRC_POST][0];
+    hop2[0] = hop2[1] = FieldRef();
+    if (post[0] == 0.0 && post[(size_t)n * h->Ls + n] == 0.0) return cudaSuccess;
+    const size_t half = half2_bytes(h);
+    FieldRef v[2];
+    for (int par = 0; par < 2; ++par) {
+        v[par].v = (char *)scratch + par * half;
+        v[par].fx = (int *)((char *)v[par].v + ((field_bytes(DWF_F64, h->Vh, 2) + 255) & ~(size_t)255));
+        hop2[par].v = (char *)scratch + (2 + par) * half;
+    }
+    cudaError_t e = launch_walls((const double *)b4, v[0], v[1], h->eo2lex, h->V, st);
+    for (int par = 0; par < 2 && e == cudaSuccess; ++par) {
+        HopArgs a = hop_args(h, DWF_F64, par, v[1 - par], hop2[par], MAT_ID);
+        a.Ls = 2;
+        a.post = h->src_mat;
+        a.post_fx = h->src_fx;
+        a.post_band = 2;
+        e = launch_hop_fx(false, a, st);
+    }
+    h->launches += 3;
+    return e;
+}
+// 1 - c (4 - M0) of the walls' rows
+void source_diagonal(const dwf_ctx *h, double y[2])
+{
+    const std::vector<double> &m = h->fm.mats[MAT_SRC_Y][0];
+    y[0] = m[0];
+    y[1] = m[(size_t)h->Ls * h->Ls - 1];
 }
 
 cudaError_t hop(dwf_ctx *h, int prec, bool dag, const HopArgs &a, cudaStream_t st)
@@ -263,7 +298,7 @@ FieldRef hop_input(const dwf_ctx *h, int prec, FieldRef f)
     return prec == DWF_F64 && h->use_fx() ? h->blocks(f) : f;
 }
 
-cudaError_t mix(dwf_ctx *h, int prec, FieldRef in, FieldRef out, int id, cudaStream_t st)
+static MixArgs mix_args(dwf_ctx *h, int prec, FieldRef in, FieldRef out, int id)
 {
     MixArgs m;
     m.in = in;
@@ -275,13 +310,32 @@ cudaError_t mix(dwf_ctx *h, int prec, FieldRef in, FieldRef out, int id, cudaStr
     m.prog = h->prog(prec, id);
     m.band = h->fm.band[id];
     m.err = h->errflag();
-    h->launches += 1;
     if (prec == DWF_F64 && h->use_fx()) {
         m.mat_fx = h->mat_fx(id);
         m.band = h->band_fx(id);
-        return launch_mix_fx(m, st);
     }
-    return launch_mix(prec, m, st);
+    return m;
+}
+
+cudaError_t mix(dwf_ctx *h, int prec, FieldRef in, FieldRef out, int id, cudaStream_t st)
+{
+    const MixArgs m = mix_args(h, prec, in, out, id);
+    h->launches += 1;
+    return m.mat_fx ? launch_mix_fx(m, st) : launch_mix(prec, m, st);
+}
+
+// x <- canonical even-odd field, xh <- M x: one kernel where the mixing is the default's
+cudaError_t pack_mix(dwf_ctx *h, int prec, const void *canon, FieldRef x, FieldRef xh, int id, cudaStream_t st)
+{
+    const MixArgs m = mix_args(h, prec, x, xh, id);
+    if (prec == DWF_F64 ? xh.fx != nullptr : m.mixmode == 0) {
+        h->launches += 1;
+        return launch_pack_mix(prec, (const double *)canon, x, m, st);
+    }
+    const cudaError_t e = launch_pack_eo(prec, (const double *)canon, x, h->Vh, h->Ls, st);
+    if (e != cudaSuccess) return e;
+    h->launches += 1;
+    return mix(h, prec, x, xh, id, st);
 }
 
 RedArgs red(dwf_ctx *h, int op, CgScalars *scal)
@@ -425,6 +479,21 @@ static int create_impl(const int dims[4], int Ls, double M0, double mf, const do
             const long long m = (long long)std::ldexp(f, B);
             mx[k] = make_int4((int)(unsigned)m, (int)(m >> 32), ex, 0);
         }
+        // the source's two walls: c / 2 of the first and the last row on the diagonal
+        double sm[8] = {0};
+        int4 sx[8];
+        for (int k = 0; k < 8; ++k) {
+            const int t = (k >> 1) & 1, row = t ? Ls - 1 : 0;
+            if (t == (k & 1)) sm[k] = h->fm.mats[MAT_SRC_POST][k >> 2][(size_t)row * Ls + row];
+            int ex = FX_ZERO;
+            const double f = sm[k] != 0.0 ? std::frexp(sm[k], &ex) : 0.0;
+            const long long m = (long long)std::ldexp(f, fx_mix_bits(2));
+            sx[k] = make_int4((int)(unsigned)m, (int)(m >> 32), ex, 0);
+        }
+        if ((e = cudaMalloc(&h->src_mat, sizeof sm)) != cudaSuccess) return fail(e, "cudaMalloc");
+        if ((e = cudaMalloc(&h->src_fx, sizeof sx)) != cudaSuccess) return fail(e, "cudaMalloc");
+        if ((e = cudaMemcpy(h->src_mat, sm, sizeof sm, cudaMemcpyHostToDevice)) != cudaSuccess) return fail(e, "cudaMemcpy");
+        if ((e = cudaMemcpy(h->src_fx, sx, sizeof sx, cudaMemcpyHostToDevice)) != cudaSuccess) return fail(e, "cudaMemcpy");
         if ((e = cudaMalloc(&h->mats_fx, mx.size() * sizeof(int4))) != cudaSuccess) return fail(e, "cudaMalloc");
         if ((e = cudaMemcpy(h->mats_fx, mx.data(), mx.size() * sizeof(int4), cudaMemcpyHostToDevice)) != cudaSuccess)
             return fail(e, "cudaMemcpy");
@@ -510,6 +579,8 @@ int dwf_destroy(dwf_handle h)
         if (h->gauge[k]) cudaFree(h->gauge[k]);
     }
     if (h->mats_fx) cudaFree(h->mats_fx);
+    if (h->src_mat) cudaFree(h->src_mat);
+    if (h->src_fx) cudaFree(h->src_fx);
     for (int k = 0; k < 2; ++k)
         if (h->progs_dev[k]) cudaFree(h->progs_dev[k]);
     if (h->nbr) cudaFree(h->nbr);
@@ -564,8 +635,7 @@ int dwf_set_gauge(dwf_handle h, const void *U, void *stream)
     if (h->slab)   // the global field, the slab's links with the global boundary phases
         CK(launch_slab_pack_gauge(h, (const double *)U, st));
     else
-        CK(launch_pack_gauge((const double *)U, h->dims, h->bc, h->eo2lex, h->nbr, h->gauge[0], h->gauge[1],
-                             h->gauge[2], st));
+        CK(launch_pack_gauge((const double *)U, h->dims, h->bc, h->gauge[0], h->gauge[1], h->gauge[2], st));
     h->launches += 1;
     h->has_gauge = true;
     return DWF_OK;
@@ -622,10 +692,9 @@ static int apply_impl(dwf_handle h, int op, int prec, const void *in, void *out,
         FieldRef x = h->field("ap_xe", prec, &e), xh = h->field("ap_he", prec, &e);
         FieldRef t = h->field("ap_ho", prec, &e), y = h->field("ap_ye", prec, &e);
         if (!x.v || !xh.v || !t.v || !y.v) return dwf_cuda_error(e, "workspace");
-        CK(launch_pack_eo(prec, (const double *)in, x, h->Vh, h->Ls, st));
-        h->launches += 2;   // pack + unpack below
+        h->launches += 1;   // unpack below
         xh = hop_input(h, prec, xh), t = hop_input(h, prec, t);
-        CK(mix(h, prec, x, xh, dag ? MAT_QT : MAT_P, st));
+        CK(pack_mix(h, prec, in, x, xh, dag ? MAT_QT : MAT_P, st));
         HopArgs a1 = hop_args(h, prec, 1, xh, t, dag ? MAT_MT : MAT_M);
         CK(hop(h, prec, dag, a1, st));
         HopArgs a2 = hop_args(h, prec, 0, t, y, dag ? MAT_NPT4 : MAT_NQ4);
@@ -681,9 +750,7 @@ int dwf_slab_apply_eo(dwf_handle h, int prec, int stage, int dag, const void *in
     FieldRef t = h->field("sl_t", prec, &e), y = h->field("sl_y", prec, &e);
     if (!x.v || !xh.v || !t.v || !y.v) return dwf_cuda_error(e, "workspace");
     if (stage == 0) {   // x^ = P x (Q^T x for the adjoint); its faces go to the neighbours
-        CK(launch_pack_eo(prec, (const double *)in, x, h->Vh, h->Ls, st));
-        h->launches += 1;
-        CK(mix(h, prec, x, xh, dag ? MAT_QT : MAT_P, st));
+        CK(pack_mix(h, prec, in, x, xh, dag ? MAT_QT : MAT_P, st));
     } else if (stage == 1) {   // t = M H_oe x^ (M^T H^dag_oe), reading x^'s ghost rows; t's faces go out
         HopArgs a1 = hop_args(h, prec, 1, xh, t, dag ? MAT_MT : MAT_M);
         CK(hop(h, prec, dag != 0, a1, st));
@@ -941,21 +1008,14 @@ int dwf_source_5d(dwf_handle h, const void *b4, void *b5, void *stream)
     if (rc) return rc;
     cudaStream_t st = (cudaStream_t)stream;
     cudaError_t e = cudaSuccess;
-    double *v5 = (double *)h->ws("src_v5", (size_t)h->V * h->Ls * 24 * 8, &e);
-    FieldRef ve = h->field("ap_xe", DWF_F64, &e), vo = h->field("ap_xo", DWF_F64, &e);
-    FieldRef oe = h->field("ap_ye", DWF_F64, &e), oo = h->field("ap_yo", DWF_F64, &e);
-    if (!v5 || !ve.v || !vo.v || !oe.v || !oo.v) return dwf_cuda_error(e, "workspace");
-    CK(launch_chiral_embed((const double *)b4, v5, h->V, h->Ls, st));
-    h->launches += 3;   // embed, pack, unpack
-    CK(launch_pack_full(DWF_F64, v5, ve, vo, h->eo2lex, h->Vh, h->V, h->Ls, st));
-    for (int par = 0; par < 2; ++par) {
-        HopArgs a = hop_args(h, DWF_F64, par, par ? ve : vo, par ? oo : oe, MAT_SRC_POST);
-        a.y = par ? vo : ve;
-        a.ymode = 2;
-        a.ymat = h->mat(DWF_F64, MAT_SRC_Y);
-        CK(hop_fp64(h, a, st));
-    }
-    CK(launch_unpack_full(DWF_F64, oe, oo, (double *)b5, h->eo2lex, h->Vh, h->V, h->Ls, st));
+    void *scratch = h->ws("src_walls", source_scratch_bytes(h), &e);
+    if (!scratch) return dwf_cuda_error(e, "workspace");
+    FieldRef hop2[2];
+    double y[2];
+    CK(source_hops(h, b4, scratch, hop2, st));
+    source_diagonal(h, y);
+    CK(launch_source_canon((const double *)b4, hop2[0], hop2[1], h->eo2lex, y[0], y[1], (double *)b5, h->V, h->Ls, st));
+    h->launches += 1;
     return DWF_OK;
 }
 

@@ -54,7 +54,7 @@ enum MatId {
     MAT_NPT4,        // -1/4 (B R)^T
     MAT_ID,          // 1
     MAT_HALF_Q,      // +1/2 R^-1 A5^-1
-    MAT_SRC_POST,    // c/2                 (hop part of 1 - c D_W, 5D source)
+    MAT_SRC_POST,    // c/2                 (hop part of 1 - c D_W; the source takes its walls' entries)
     MAT_SRC_Y,       // 1 - c (4 - M0)      (diagonal part of 1 - c D_W)
     MAT_NQUARTER,    // -1/4                (second even-odd form)
     MAT_NMT4,        // -1/4 (B A5^-1)^T    (its adjoint)
@@ -204,6 +204,9 @@ cudaError_t launch_unpack_full(int prec, FieldRef even, FieldRef odd, double *ca
 cudaError_t launch_pack_eo(int prec, const double *canon, FieldRef f, int Vh, int Ls, cudaStream_t st);
 cudaError_t launch_unpack_eo(int prec, FieldRef f, double *canon, int Vh, int Ls, cudaStream_t st);
 
+// pack_eo into x and a.out = M x in one pass (FP64: a.out a block field; else a.mixmode 0)
+cudaError_t launch_pack_mix(int prec, const double *canon, FieldRef x, const MixArgs &a, cudaStream_t st);
+
 // precision conversion between internal fields of the same parity
 cudaError_t launch_convert(int prec_in, FieldRef in, int prec_out, FieldRef out, int Vh, int Ls, cudaStream_t st);
 // x64 += xs (xs: FP64 if xs_prec == DWF_F64 else FP32); then xs = 0
@@ -217,12 +220,19 @@ cudaError_t launch_zero(int prec, FieldRef f, int Vh, int Ls, cudaStream_t st);
 
 // gauge and index tables
 cudaError_t launch_build_tables(const int dims[4], int *nbr, int *eo2lex, cudaStream_t st);
-cudaError_t launch_pack_gauge(const double *U, const int dims[4], const int bc[4], const int *eo2lex,
-                              const int *nbr, void *g64, void *g32, void *g16, cudaStream_t st);
+cudaError_t launch_pack_gauge(const double *U, const int dims[4], const int bc[4], void *g64, void *g32, void *g16,
+                              cudaStream_t st);
 
-// 4D source / projection on canonical 5D fields (FP64)
+// projection on canonical 5D fields (FP64)
 cudaError_t launch_project4d(const double *x5, double *x4, int V, int Ls, cudaStream_t st);
-cudaError_t launch_chiral_embed(const double *b4, double *b5, int V, int Ls, cudaStream_t st);
+// The 5D source (dwf_source_5d): P_+ b4 and P_- b4 as block fields of two slices per
+// parity; after the hop on those (fields of two FP64 slices he, ho, null for none),
+// the source as a canonical field or as one half.
+cudaError_t launch_walls(const double *b4, FieldRef even, FieldRef odd, const int *eo2lex, int V, cudaStream_t st);
+cudaError_t launch_source_canon(const double *b4, FieldRef he, FieldRef ho, const int *eo2lex, double y0, double y1,
+                                double *b5, int V, int Ls, cudaStream_t st);
+cudaError_t launch_source_half(const double *b4, FieldRef hf, const int *eo2lex_par, double y0, double y1, FieldRef f,
+                               int Vh, int Ls, cudaStream_t st);
 
 // bytes of one internal half field
 size_t field_bytes(int prec, int Vh, int Ls);
@@ -292,6 +302,9 @@ struct dwf_ctx {
     void *mats_dev[3] = {nullptr, nullptr, nullptr};   // double / float / float copies (F16 uses float)
     void *mats_fx = nullptr;                           // int4 [MAT_COUNT][2][Ls][Ls]: fixed-point constants
     const int4 *mat_fx(int id) const { return (const int4 *)mats_fx + (size_t)2 * Ls * Ls * id; }
+    // the source's hop on two slices: c / 2 of rows 1 and Ls, as [2][2][2] doubles and constants
+    double *src_mat = nullptr;
+    int4 *src_fx = nullptr;
     int band_fx(int id) const { return fm.diag[id] ? 2 : (fm.band[id] ? 1 : 0); }
     // the FP64 operator runs on fixed-point blocks unless the caller chose an FP64 hop
     // variant or mixing mode of its own

@@ -22,7 +22,7 @@ using namespace dwf;
 namespace dwf_detail {
 HopArgs hop_args(dwf_ctx *h, int prec, int out_par, FieldRef in, FieldRef out, int post);
 cudaError_t hop(dwf_ctx *h, int prec, bool dag, const HopArgs &a, cudaStream_t st);
-cudaError_t mix(dwf_ctx *h, int prec, FieldRef in, FieldRef out, int id, cudaStream_t st);
+cudaError_t pack_mix(dwf_ctx *h, int prec, const void *canon, FieldRef x, FieldRef xh, int id, cudaStream_t st);
 FieldRef hop_input(const dwf_ctx *h, int prec, FieldRef f);
 }  // namespace dwf_detail
 using namespace dwf_detail;
@@ -94,9 +94,7 @@ extern "C" int dwf_apply_eo_noalloc(dwf_handle h, int prec, int dag, const void 
         t.fx = xh.fx + (size_t)h->Vh * h->Ls;
     }
     cudaStream_t st = (cudaStream_t)stream;
-    if ((e = launch_pack_eo(prec, (const double *)in, x, h->Vh, h->Ls, st)) != cudaSuccess)
-        return dwf_cuda_error(e, "pack");
-    if ((e = mix(h, prec, x, xh, dag ? MAT_QT : MAT_P, st)) != cudaSuccess) return dwf_cuda_error(e, "mix");
+    if ((e = pack_mix(h, prec, in, x, xh, dag ? MAT_QT : MAT_P, st)) != cudaSuccess) return dwf_cuda_error(e, "pack");
     HopArgs a1 = hop_args(h, prec, 1, xh, t, dag ? MAT_MT : MAT_M);
     if ((e = hop(h, prec, dag != 0, a1, st)) != cudaSuccess) return dwf_cuda_error(e, "hop");
     HopArgs a2 = hop_args(h, prec, 0, t, y, dag ? MAT_NPT4 : MAT_NQ4);
@@ -105,6 +103,6 @@ extern "C" int dwf_apply_eo_noalloc(dwf_handle h, int prec, int dag, const void 
     if ((e = hop(h, prec, dag != 0, a2, st)) != cudaSuccess) return dwf_cuda_error(e, "hop");
     if ((e = launch_unpack_eo(prec, y, (double *)out, h->Vh, h->Ls, st)) != cudaSuccess)
         return dwf_cuda_error(e, "unpack");
-    h->launches += 2;   // pack and unpack (mix and hop count their own launches)
+    h->launches += 1;   // unpack (pack_mix and hop count their own launches)
     return DWF_OK;
 }

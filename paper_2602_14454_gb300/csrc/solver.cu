@@ -36,7 +36,9 @@ HopArgs hop_args(dwf_ctx *h, int prec, int out_par, FieldRef in, FieldRef out, i
 HopArgs with_programs(dwf_ctx *h, int prec, const HopArgs &a0);
 cudaError_t hop(dwf_ctx *h, int prec, bool dag, const HopArgs &a, cudaStream_t st);
 cudaError_t hop_cg_plain(dwf_ctx *h, int prec, bool dag, const HopArgs &a, cudaStream_t st);
-cudaError_t hop_fp64(dwf_ctx *h, const HopArgs &a, cudaStream_t st);
+size_t source_scratch_bytes(const dwf_ctx *h);
+cudaError_t source_hops(dwf_ctx *h, const void *b4, void *scratch, FieldRef hop2[2], cudaStream_t st);
+void source_diagonal(const dwf_ctx *h, double y[2]);
 cudaError_t mix(dwf_ctx *h, int prec, FieldRef in, FieldRef out, int id, cudaStream_t st);
 FieldRef hop_input(const dwf_ctx *h, int prec, FieldRef f);
 RedArgs red(dwf_ctx *h, int op, CgScalars *scal);
@@ -696,7 +698,9 @@ size_t system_bytes(const dwf_ctx *h, int ps)
            round256(sizeof(CgUpdateArgs)) + 4 * round256(sizeof(HopArgs));
 }
 
-size_t shared_bytes(int V, int Vh, int Ls) { return 6 * field_total(DWF_F64, Vh, Ls) + round256((size_t)V * Ls * 24 * 8); }
+// the canonical buffer of a wave: a 5D field, or the source's scratch where that is larger (Ls < 5)
+size_t canon_bytes(const dwf_ctx *h, int Ls) { return std::max((size_t)h->V * Ls * 24 * 8, source_scratch_bytes(h)); }
+size_t shared_bytes(const dwf_ctx *h, int Ls) { return 6 * field_total(DWF_F64, h->Vh, Ls) + round256(canon_bytes(h, Ls)); }
 
 struct SysRun {
     dwf_ctx *h = nullptr;
@@ -712,22 +716,18 @@ struct SysRun {
 
 // (b_e, b_o) = even / odd halves of b5 = (1 - c D_W) P^dag (0, .., b4) in the
 // internal FP64 layout (the source of Sec. 2.2, as dwf_source_5d), using the
-// canonical buffer v5 and the temporaries ve, vo.
-cudaError_t source_eo(dwf_ctx *h, const void *b4, double *v5, FieldRef ve, FieldRef vo, FieldRef be, FieldRef bo,
-                      cudaStream_t st)
+// canonical buffer v5 (canon_bytes).
+cudaError_t source_eo(dwf_ctx *h, const void *b4, double *v5, FieldRef be, FieldRef bo, cudaStream_t st)
 {
-    cudaError_t e;
-    if ((e = launch_chiral_embed((const double *)b4, v5, h->V, h->Ls, st)) != cudaSuccess) return e;
-    if ((e = launch_pack_full(DWF_F64, v5, ve, vo, h->eo2lex, h->Vh, h->V, h->Ls, st)) != cudaSuccess) return e;
+    FieldRef hop2[2];
+    double y[2];
+    cudaError_t e = source_hops(h, b4, v5, hop2, st);
+    source_diagonal(h, y);
+    for (int par = 0; par < 2 && e == cudaSuccess; ++par)
+        e = launch_source_half((const double *)b4, hop2[par], h->eo2lex + (size_t)par * h->Vh, y[0], y[1], par ? bo : be,
+                               h->Vh, h->Ls, st);
     h->launches += 2;
-    for (int par = 0; par < 2; ++par) {
-        HopArgs a = hop_args(h, DWF_F64, par, par ? ve : vo, par ? bo : be, MAT_SRC_POST);
-        a.y = par ? vo : ve;
-        a.ymode = 2;
-        a.ymat = h->mat(DWF_F64, MAT_SRC_Y);
-        if ((e = hop_fp64(h, a, st)) != cudaSuccess) return e;
-    }
-    return cudaSuccess;
+    return e;
 }
 
 // FP64 true residual; convergence test; else the normal residual in the inner
@@ -775,7 +775,7 @@ int sys_prepare(SysRun &R, const void *b4, double *v5, const dwf_solve_params *p
 {
     dwf_ctx *h = R.h;
     Bufs &B = R.B;
-    CK(source_eo(h, b4, v5, B.r64, B.t64, B.be, B.bo, st));
+    CK(source_eo(h, b4, v5, B.be, B.bo, st));
     CK(launch_norm2(DWF_F64, B.be, h->Vh, h->Ls, red(h, RED_STORE, B.n64), st));
     CK(launch_norm2(DWF_F64, B.bo, h->Vh, h->Ls, red(h, RED_STORE, B.aux), st));
     h->launches += 2;
@@ -820,7 +820,7 @@ int sys_finish(SysRun &R, const void *b4, void *x4, double *v5, const dwf_solve_
 {
     dwf_ctx *h = R.h;
     Bufs &B = R.B;
-    CK(source_eo(h, b4, v5, B.r64, B.t64, B.be, B.bo, st));
+    CK(source_eo(h, b4, v5, B.be, B.bo, st));
     const FieldRef xh = hop_input(h, DWF_F64, B.h64), t = hop_input(h, DWF_F64, B.t64);
     CK(mix(h, DWF_F64, B.x64, xh, MAT_P, st));
     {
@@ -912,7 +912,7 @@ int batch_impl(dwf_handle const *hs_in, const void *const *b4, void *const *x4, 
     long long launches0 = 0;
     for (dwf_ctx *h : uniq_handles) launches0 += h->launches;
     const int V = h0->V, Vh = h0->Vh;
-    const size_t shared = shared_bytes(V, Vh, Lsmax);
+    const size_t shared = shared_bytes(h0, Lsmax);
     size_t freeb = 0, totalb = 0;
     CK(cudaMemGetInfo(&freeb, &totalb));
     const size_t reserve = std::max((size_t)2 << 30, totalb / 20);
@@ -985,7 +985,7 @@ int batch_impl(dwf_handle const *hs_in, const void *const *b4, void *const *x4, 
         FieldRef be = A.field(DWF_F64, Vh, Lsmax), bo = A.field(DWF_F64, Vh, Lsmax);
         FieldRef r64 = A.field(DWF_F64, Vh, Lsmax), t64 = A.field(DWF_F64, Vh, Lsmax);
         FieldRef h64 = A.field(DWF_F64, Vh, Lsmax), xo64 = A.field(DWF_F64, Vh, Lsmax);
-        double *v5 = (double *)A.take((size_t)V * Lsmax * 24 * 8);
+        double *v5 = (double *)A.take(canon_bytes(h0, Lsmax));
         int *skip_dev = (int *)A.take(sizeof(int) * (size_t)nw);
         if (!v5 || !skip_dev || !xo64.v) {
             cleanup();
