@@ -360,8 +360,8 @@ long long dwf_launch_count(dwf_handle h);
  * thread's slices; variant 7 (FP32/FP16, dense mixing, Ls a multiple of 4) is
  * a persistent kernel of sb-site tiles with the tile's links staged in shared
  * memory one tile ahead and the mixing done by half of the threads, two
- * outputs each; variant 9 (FP32/FP16, dense mixing, Ls dividing 32 and a
- * multiple of 4) is persistent and warp-autonomous: every warp walks its own
+ * outputs each; variant 9 (FP32, or FP16 with Ls dividing 32 and a
+ * multiple of 4; dense mixing) is persistent and warp-autonomous: every warp walks its own
  * tiles of 32/Ls sites (a window sweeping the lattice, see dwf_set_sweep) with
  * its own shared-memory links (staged one tile ahead) and mixing tile, and no
  * CTA barrier; there sb counts warps per CTA (1..4) and ns selects the

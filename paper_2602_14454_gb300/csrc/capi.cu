@@ -278,18 +278,27 @@ cudaError_t hop(dwf_ctx *h, int prec, bool dag, const HopArgs &a, cudaStream_t s
     return launch_hop(prec, dag, with_programs(h, prec, a), h->hop_var[prec], h->hop_ns[prec], h->hop_sb[prec], st);
 }
 
-// The CG iteration's K_a and K_c (the hops whose only mixing is the dense M or
-// M^T) in FP32 take the structured mixing by register chains when the caller
-// left the mixing mode and the hop variant at their defaults (variant 9, Ls 8
-// or 16): 3-4 % faster than the dense form for those two launches at 32^3x64,
-// Ls 16, where the banded K_d and the two-matrix K_b are not.
-cudaError_t hop_cg_plain(dwf_ctx *h, int prec, bool dag, const HopArgs &a, cudaStream_t st)
+// A hop of the CG iteration.  In FP32, when the caller left the mixing mode and the
+// hop variant at their defaults, the hops that mix with inverses only (K_a, K_b, K_c)
+// take the structured mixing by register chains at Ls 12 and 16: it reads every tile
+// element once where the dense form reads the site's tile and a matrix row per
+// output.  24^3x48, chains against dense: Ls 16 K_a 372 / 426 us, K_b 533 / 591 us;
+// Ls 12 338 / 380, 472 / 515; at Ls 8 the dense form wins (K_a 190 / 186, K_b
+// 261 / 240).  The banded K_d reads three rows per output and stays dense (449 / 578).
+HopArgs cg_programs(dwf_ctx *h, int prec, const HopArgs &a)
 {
-    const bool chains = prec == DWF_F32 && h->mixmode[prec] < 0 && h->fm.structured && (h->Ls == 8 || h->Ls == 16) &&
-                        (h->hop_var[prec] < 0 || h->hop_var[prec] == 9) && !a.ymode && !a.zmat && !a.rin.v;
-    if (!chains) return hop(h, prec, dag, a, st);
+    if (prec == DWF_F32 && h->mixmode[prec] < 0 && h->fm.structured && (h->Ls == 12 || h->Ls == 16) &&
+        (h->hop_var[prec] < 0 || h->hop_var[prec] == 9) && a.ymode != 2 && !a.rin.v) {
+        const HopArgs c = with_programs_mode(h, prec, a, 1);
+        if (!c.post_band && !(c.zmat && c.z_band)) return c;
+    }
+    return with_programs(h, prec, a);
+}
+cudaError_t hop_cg(dwf_ctx *h, int prec, bool dag, const HopArgs &a, cudaStream_t st)
+{
+    if (prec == DWF_F64) return hop(h, prec, dag, a, st);
     h->launches += 1;
-    return launch_hop(prec, dag, with_programs_mode(h, prec, a, 1), 9, h->hop_ns[prec], h->hop_sb[prec], st);
+    return launch_hop(prec, dag, cg_programs(h, prec, a), h->hop_var[prec], h->hop_ns[prec], h->hop_sb[prec], st);
 }
 
 // A field that only hops and mixings read: FP64 fields are kept as blocks then.
@@ -1217,9 +1226,9 @@ int dwf_autotune(dwf_handle h, int prec, const char *cache_path, void *stream)
                 if (var == 1 || var == 2 || var == 6 || var == 8) continue;   // numbers not in use
                 if (mix != 0 && var != 0) continue;   // those mixings exist in the direct variant only
                 if (var == 5 && prec != DWF_F16) continue;
-                if ((var == 7 || var == 9) && (prec == DWF_F64 || h->Ls % 4 != 0)) continue;
-                if (var == 7 && ns != 1) continue;
-                if (var == 9 && (32 % h->Ls != 0 || ns > 2)) continue;
+                if ((var == 7 || var == 9) && prec == DWF_F64) continue;
+                if (var == 7 && (ns != 1 || h->Ls % 4 != 0)) continue;
+                if (var == 9 && (ns > 2 || (prec == DWF_F16 && (h->Ls % 4 != 0 || 32 % h->Ls != 0)))) continue;
                 if (ns == 4 && var != 5) continue;
                 if (var != 9 && h->Ls % ns) continue;
                 const int LsN = h->Ls / (var == 9 ? 1 : ns);

@@ -189,7 +189,7 @@ cudaError_t launch_mix_tc(int prec, const MixArgs &a, cudaStream_t st);
 cudaError_t launch_cg_update(int prec, const CgUpdateArgs &a, cudaStream_t st);
 // Batched launches over nsys systems with equal Ls (tables in device memory;
 // a0: host copy of one entry, for Ls, Vh and the mixing mode): the direct hop
-// with (ns, sb) tiling, and the CG update.
+// with (ns, sb) tiling (sb < 0: the FP32 default variant), and the CG update.
 cudaError_t launch_hop_batch(int prec, bool dag, const HopArgs *tab, int nsys, const HopArgs &a0, int ns, int sb,
                              cudaStream_t st);
 cudaError_t launch_cg_update_batch(int prec, const CgUpdateArgs *tab, int nsys, const CgUpdateArgs &a0,

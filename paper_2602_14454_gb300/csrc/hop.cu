@@ -21,9 +21,10 @@ cudaError_t launch_hop_fx(bool dag, const HopArgs &a, cudaStream_t st)
 // Defaults from the sweeps on GB300 at 16^3x32 and 32^3x64, Ls 16: FP32 the
 // warp-autonomous variant 9 (83.7 / 1446 us per hop against 102.4 / 1519 us for
 // the direct variant 0; the whole FP32 CG iteration 475 / 7897 us against
-// 586 / 8755 us), FP16 variant 5 (84.7 / 1183 us; variant 9: 87.8 / 1372 us),
-// FP64 variant 0.  Variant 9 needs dense mixing and Ls dividing 32 (and a
-// multiple of 4); otherwise the FP32 default is variant 0.
+// 586 / 8755 us), FP16 variant 5 (84.7 / 1183 us; variant 9: 87.8 / 1372 us).
+// Variant 9 takes dense mixing (FP32 any Ls; FP16 Ls dividing 32 and a multiple of
+// 4) or chains (Ls 8 and 16, FP32 also 12); otherwise the default is variant 0 (FP32)
+// or 5.  FP64 answers 0 here: its default is the fixed-point hop (launch_hop_fx).
 int hop_default_variant(int prec) { return prec == DWF_F16 ? 5 : (prec == DWF_F32 ? 9 : 0); }
 
 int hop_default_ns(int prec, int Ls)
@@ -46,6 +47,11 @@ cudaError_t launch_hop_batch(int prec, bool dag, const HopArgs *tab, int nsys, c
                              cudaStream_t st)
 {
     if (nsys < 1) return cudaSuccess;
+    // SB < 0: FP32 systems on the default variant, which take its warp-autonomous form
+    // together (dense mixing, or chains where launch_hop has them)
+    if (SB < 0 && prec == DWF_F32 && (a0.mixmode == 0 || (a0.mixmode == 1 && (a0.Ls == 8 || a0.Ls == 12 || a0.Ls == 16))))
+        return dag ? hop_batch_launch_pd<DWF_F32, true>(tab, nsys, a0, 0, 0, st)
+                   : hop_batch_launch_pd<DWF_F32, false>(tab, nsys, a0, 0, 0, st);
     if (NS <= 0 || NS > 2 || (a0.Ls % NS) != 0) NS = hop_default_ns(prec, a0.Ls);
     if (SB <= 0) SB = hop_default_sb(prec, a0.Ls, NS);
     if ((a0.Ls / NS) * SB > 256) SB = 256 / (a0.Ls / NS);
@@ -79,8 +85,8 @@ cudaError_t launch_hop(int prec, bool dag, const HopArgs &a, int var, int NS, in
     // variants 7 and 9 need FP32/FP16 fields and dense mixing (9 also Ls dividing 32), else the default
     const bool v_ok = prec != DWF_F64 && a.mixmode == 0 && a.Ls % 4 == 0;
     const bool v9_ok = prec != DWF_F64 &&
-                       ((a.mixmode == 0 && a.Ls % 4 == 0 && a.Ls <= 32 && 32 % a.Ls == 0) ||
-                        (a.mixmode == 1 && (a.Ls == 8 || a.Ls == 16)));   // structured mixing: chains in registers
+                       ((a.mixmode == 0 && (prec == DWF_F32 || (a.Ls % 4 == 0 && 32 % a.Ls == 0))) ||
+                        (a.mixmode == 1 && (a.Ls == 8 || a.Ls == 16 || (prec == DWF_F32 && a.Ls == 12))));   // structured mixing: chains in registers
     if ((var == 7 && !v_ok) || (var == 9 && !v9_ok)) {
         var = prec == DWF_F16 ? 5 : 0;
         SB = 0;

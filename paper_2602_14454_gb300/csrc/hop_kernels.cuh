@@ -996,8 +996,10 @@ __global__ void __launch_bounds__(256, MINB) hop_lean_kernel(const HopArgs a)
 }
 
 // ------------------------------------------ variant 9: warp-autonomous hop
-// Every warp works alone on its own tiles of 32 / Ls sites (Ls dividing 32),
-// persistent over its CTA's contiguous range of tiles, with no CTA barrier
+// Every warp works alone on its own tiles of 32 / Ls sites (where Ls does not divide
+// 32, FP32 only, the last 32 mod Ls lanes idle: the load/store path, not the issue
+// slots, bounds it; 24^3x48, Ls 12: 380 us per dense hop against 408 us direct, whole
+// iterations 1888 / 2291 us; 16^3x32, Ls 10: 65 / 80 us, 357 / 438 us), persistent over its CTA's contiguous range of tiles, with no CTA barrier
 // after the matrices are loaded: the warp's links (its sites' 8 directions)
 // are copied into its own shared-memory buffer with 16-byte asynchronous
 // copies one tile ahead (warp barrier only) and read as 16-byte vectors; the
@@ -1011,7 +1013,8 @@ __host__ __device__ constexpr size_t wa_warp_bytes(int Ls)
 {
     return (size_t)2 * (32 / Ls) * LeanGeom<P>::LINK_BYTES + (size_t)(32 / Ls) * (Ls * 14 + 12) * sizeof(float2);
 }
-__host__ __device__ constexpr int wa_mat_row(int Ls) { return ((Ls / 4) & 1) ? Ls : Ls + 4; }
+// floats between matrix rows: an odd number of 16-byte vectors
+__host__ __device__ constexpr int wa_mat_row(int Ls) { return 4 * (((Ls + 3) / 4) | 1); }
 // the CTA's front area: the three dense matrices, then the three structured
 // programs (at most 2048 bytes, checked where they are defined)
 __host__ __device__ constexpr size_t wa_front_bytes(int Ls)
@@ -1054,6 +1057,7 @@ __device__ __forceinline__ void wa_mix(const float *M, const float2 *site_tile, 
         const float ca[4] = {a4.x, a4.y, a4.z, a4.w}, cb[4] = {b4.x, b4.y, b4.z, b4.w};
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
+            if (t0 + k >= Ls) break;
             const float2 cu = p_splat(ca[k]), cl = p_splat(cb[k]);
             const float4 *row = base + (size_t)(t0 + k) * (LEAN_ROW / 2);
 #pragma unroll
@@ -1081,7 +1085,7 @@ __device__ __forceinline__ void wa_mix(const float *M, const float2 *site_tile, 
 // The sites of a warp tile lie wc_site_stride floats apart: 24 banks on, so
 // the 32 chains a warp loads at once (24 components of one site, 8 of the
 // next) hit distinct banks.
-__host__ __device__ constexpr int wc_site_stride(int Ls) { return Ls * 14 + 12; }   // float2
+__host__ __device__ constexpr int wc_site_stride(int Ls) { return Ls * 14 + (28 - Ls * 14 % 16) % 16; }   // float2
 
 // a program in shared memory with the chirality-interleaved d vectors
 struct WcProg {
@@ -1194,7 +1198,7 @@ __device__ __forceinline__ void wc_take(const float2 *row, float2 *o)
 // (every lane of the warp calls it; progs: post, y, z)
 template <int P, int LS>
 __device__ __forceinline__ float wc_epilogue(const HopArgs &a, const float2 *acc, float2 *tile, const WcProg *progs,
-                                             int j, int s, int site, bool active, int lane)
+                                             int j, int s, int site, bool worker, bool active, int lane)
 {
     float2 *row = tile + (size_t)j * wc_site_stride(LS) + (size_t)s * LEAN_ROW;
     float *tf = reinterpret_cast<float *>(tile);
@@ -1209,7 +1213,7 @@ __device__ __forceinline__ float wc_epilogue(const HopArgs &a, const float2 *acc
         for (int k = 0; k < 12; ++k) xv[k] = p_fma(xa, dx[k], xv[k]);
         st_pairs_cs<DWF_F32>(xf, (size_t)site, s, LS, xv);
     }
-    lean_put(row, acc);   // inactive lanes put zeros
+    if (worker) lean_put(row, acc);   // sites beyond the last put zeros
     __syncwarp();
     float2 o[12];
     wc_chains<LS>(progs, tf, lane);
@@ -1222,7 +1226,7 @@ __device__ __forceinline__ float wc_epilogue(const HopArgs &a, const float2 *acc
         if (active) ld_pairs_cs<P>(a.y, (size_t)site, s, LS, y);
         if (a.ymode == 2) {
             __syncwarp();
-            lean_put(row, y);
+            if (worker) lean_put(row, y);
             __syncwarp();
             wc_chains<LS>(progs + 1, tf, lane);
             __syncwarp();
@@ -1247,7 +1251,7 @@ __device__ __forceinline__ float wc_epilogue(const HopArgs &a, const float2 *acc
     }
     if (a.zmat) {
         __syncwarp();
-        lean_put(row, o);
+        if (worker) lean_put(row, o);
         __syncwarp();
         wc_chains<LS>(progs + 2, tf, lane);
         __syncwarp();
@@ -1348,13 +1352,16 @@ __device__ __forceinline__ void wa_issue_links(const void *gauge, int site0, int
 // t-slice away are still in L2 when those are processed (which a contiguous
 // range per CTA, spreading the tiles in work over the whole lattice, loses once
 // the fields exceed L2).
-template <int P, bool DAG, int MINB, int MIX>
-__global__ void __launch_bounds__(128, MINB) hop_wa_kernel(const HopArgs a)
+// bid of nb: this CTA among those that work on a's lattice.
+template <int P, bool DAG, int MIX>
+__device__ __forceinline__ void hop_wa_body(const HopArgs &a, int bid, int nb)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int Ls = a.Ls, SPW = 32 / Ls;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
-    const int j = lane / Ls, s = lane - (lane / Ls) * Ls;
+    // Ls need not divide 32: the lanes beyond the last whole site idle
+    const int j = lane / Ls < SPW ? lane / Ls : 0, s = lane - (lane / Ls) * Ls;
+    const bool worker = lane < SPW * Ls;
     const int MR = wa_mat_row(Ls), msz = 2 * Ls * MR;
     float *mats = reinterpret_cast<float *>(smem_raw);
     // MIX 1: the structured programs, after the matrix area
@@ -1385,13 +1392,13 @@ __global__ void __launch_bounds__(128, MINB) hop_wa_kernel(const HopArgs a)
     __syncthreads();   // the matrices (the only CTA barrier before the final reduction)
 
     const int ntiles = (a.Vh + SPW - 1) / SPW;
-    const int G = gridDim.x * nwarps;
+    const int G = nb * nwarps;
     float nrm = 0.f;
-    int u = blockIdx.x * nwarps + warp;
+    int u = bid * nwarps + warp;
     if (u < ntiles) wa_issue_links<P>(a.gauge, sweep_site(a, u * SPW), min(SPW, a.Vh - u * SPW), links, lane);
     for (int k = 0; u < ntiles; ++k, u += G) {
         const int site = sweep_site(a, u * SPW) + j;
-        const bool active = u * SPW + j < a.Vh;
+        const bool active = worker && u * SPW + j < a.Vh;
         int n8[8];
         if (active) {
             const int4 *p = reinterpret_cast<const int4 *>(a.nbr + (size_t)site * 8);
@@ -1420,15 +1427,39 @@ __global__ void __launch_bounds__(128, MINB) hop_wa_kernel(const HopArgs a)
             lean_dir<P, DAG, 7>(acc, a.in, n8[7], s, Ls, lk);
         }
         if constexpr (MIX == 1) {
-            if (Ls == 16) nrm += wc_epilogue<P, 16>(a, acc, tile, progs, j, s, site, active, lane);
-            else nrm += wc_epilogue<P, 8>(a, acc, tile, progs, j, s, site, active, lane);   // Ls 8 (launch_pd)
+            if (Ls == 16) nrm += wc_epilogue<P, 16>(a, acc, tile, progs, j, s, site, worker, active, lane);
+            else if (Ls == 12) nrm += wc_epilogue<P, 12>(a, acc, tile, progs, j, s, site, worker, active, lane);
+            else nrm += wc_epilogue<P, 8>(a, acc, tile, progs, j, s, site, worker, active, lane);   // Ls 8 (launch_pd)
         } else {
             nrm += wa_epilogue<P>(a, acc, site_tile, mats, s, site, active);
         }
     }
     cp_async_wait<0>();
-    if (a.red.op != RED_NONE) grid_reduce(nrm, a.red);
+    if (a.red.op != RED_NONE) grid_reduce(nrm, a.red, (unsigned)bid, (unsigned)nb);
 }
+
+template <int P, bool DAG, int MINB, int MIX>
+__global__ void __launch_bounds__(128, MINB) hop_wa_kernel(const HopArgs a)
+{
+    hop_wa_body<P, DAG, MIX>(a, blockIdx.x, gridDim.x);
+}
+
+// Batched form (FP32): CTA b belongs to system b % nsys, whose matrices it loads, and
+// walks that system's tiles with the system's other CTAs; as many CTAs in all as the
+// device holds.  8^3x16, 18 systems of Ls 8, 12 and 16: 24-44 us a hop of one Ls
+// against 44 us in the direct form, the whole batch 105 ms (128).
+template <bool DAG, int MIX>
+__global__ void __launch_bounds__(128, 4) hop_wa_batch_kernel(const HopArgs *__restrict__ tab, int nsys)
+{
+    __shared__ __align__(16) unsigned char abuf[sizeof(HopArgs)];
+    const unsigned *src = reinterpret_cast<const unsigned *>(tab + blockIdx.x % nsys);
+    for (int k = threadIdx.x; k < (int)(sizeof(HopArgs) / 4); k += blockDim.x) reinterpret_cast<unsigned *>(abuf)[k] = src[k];
+    __syncthreads();
+    const HopArgs &a = *reinterpret_cast<const HopArgs *>(abuf);
+    if (a.skip && *a.skip) return;
+    hop_wa_body<DWF_F32, DAG, MIX>(a, blockIdx.x / nsys, gridDim.x / nsys);
+}
+
 
 
 // ---------------------------------------------------------------- variant 10
@@ -1797,9 +1828,33 @@ cudaError_t launch_direct_batch(const HopArgs *tab, int nsys, const HopArgs &a0,
     return cudaGetLastError();
 }
 
+template <bool DAG, int MIX>
+cudaError_t launch_wa_batch(const HopArgs *tab, int nsys, const HopArgs &a0, cudaStream_t st)
+{
+    static unsigned long long optin = 0;
+    int dev = 0, nsm = 0, per_sm = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    if ((e = smem_optin(hop_wa_batch_kernel<DAG, MIX>, 200 * 1024, optin)) != cudaSuccess) return e;
+    if ((e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
+    constexpr int nw = 4;
+    const size_t smem = wa_cta_bytes<DWF_F32>(a0.Ls, nw);
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, hop_wa_batch_kernel<DAG, MIX>, 32 * nw, smem);
+    if (e != cudaSuccess) return e;
+    if (per_sm < 1) per_sm = 1;
+    const int SPW = 32 / a0.Ls, most = ((a0.Vh + SPW - 1) / SPW + nw - 1) / nw;
+    int each = nsm * per_sm / nsys;   // CTAs per system
+    each = each < 1 ? 1 : each > most ? most : each;
+    hop_wa_batch_kernel<DAG, MIX><<<(unsigned)each * nsys, 32 * nw, smem, st>>>(tab, nsys);
+    return cudaGetLastError();
+}
+
 template <int P, bool DAG>
 cudaError_t launch_batch_pd(const HopArgs *tab, int nsys, const HopArgs &a0, int NS, int SB, cudaStream_t st)
 {
+    if constexpr (P == DWF_F32) {   // NS 0: warp-autonomous (launch_hop_batch)
+        if (NS == 0) return a0.mixmode == 1 ? launch_wa_batch<DAG, 1>(tab, nsys, a0, st) : launch_wa_batch<DAG, 0>(tab, nsys, a0, st);
+    }
     if constexpr (P == DWF_F16) {   // FP16 arithmetic (as hop variant 5) with dense mixing
         if (a0.mixmode == 0)
             return NS == 2 ? launch_direct_batch<P, DAG, 2, 0, true>(tab, nsys, a0, SB, st)
@@ -1932,7 +1987,9 @@ cudaError_t launch_wa(const HopArgs &a, int nw, cudaStream_t st)
     const int ntiles = (a.Vh + SPW - 1) / SPW;
     int grid = nsm * per_sm;
     if (grid > (ntiles + nw - 1) / nw) grid = (ntiles + nw - 1) / nw;
-    hop_wa_kernel<P, DAG, MINB, MIX><<<grid, 32 * nw, smem, st>>>(a);
+    HopArgs b = a;
+    if (b.zblock > 0 && (b.zblock * b.ext[0] * b.ext[1]) % SPW) b.zblock = 0;   // a tile would straddle two runs
+    hop_wa_kernel<P, DAG, MINB, MIX><<<grid, 32 * nw, smem, st>>>(b);
     return cudaGetLastError();
 }
 
@@ -1998,10 +2055,10 @@ cudaError_t launch_pd(const HopArgs &a, int var, int NS, int SB, cudaStream_t st
     // multiple of 4); SB = warps per CTA, NS selects the register budget (1: 5 CTAs of 4
     // warps per SM, 2: 4)
     if constexpr (P != DWF_F64) {
-        if (var == 9 && a.mixmode == 0 && a.Ls <= 32 && 32 % a.Ls == 0 && a.Ls % 4 == 0)
+        if (var == 9 && a.mixmode == 0 && (P == DWF_F32 || (32 % a.Ls == 0 && a.Ls % 4 == 0)))
             return NS == 2 ? launch_wa<P, DAG, 4, 0>(a, SB, st) : launch_wa<P, DAG, 5, 0>(a, SB, st);
         // structured mixing by chains in registers (Ls 8 and 16)
-        if (var == 9 && a.mixmode == 1 && (a.Ls == 8 || a.Ls == 16))
+        if (var == 9 && a.mixmode == 1 && (a.Ls == 8 || a.Ls == 16 || (P == DWF_F32 && a.Ls == 12)))
             return NS == 2 ? launch_wa<P, DAG, 4, 1>(a, SB, st) : launch_wa<P, DAG, 5, 1>(a, SB, st);
     }
     if (var == 9) var = P == DWF_F16 ? 5 : 0;

@@ -34,8 +34,9 @@ using namespace dwf;
 namespace dwf_detail {
 HopArgs hop_args(dwf_ctx *h, int prec, int out_par, FieldRef in, FieldRef out, int post);
 HopArgs with_programs(dwf_ctx *h, int prec, const HopArgs &a0);
+HopArgs cg_programs(dwf_ctx *h, int prec, const HopArgs &a);
 cudaError_t hop(dwf_ctx *h, int prec, bool dag, const HopArgs &a, cudaStream_t st);
-cudaError_t hop_cg_plain(dwf_ctx *h, int prec, bool dag, const HopArgs &a, cudaStream_t st);
+cudaError_t hop_cg(dwf_ctx *h, int prec, bool dag, const HopArgs &a, cudaStream_t st);
 size_t source_scratch_bytes(const dwf_ctx *h);
 cudaError_t source_hops(dwf_ctx *h, const void *b4, void *scratch, FieldRef hop2[2], cudaStream_t st);
 void source_diagonal(const dwf_ctx *h, double y[2]);
@@ -181,9 +182,7 @@ cudaError_t inner_iteration(dwf_ctx *h, const Bufs &B, cudaStream_t st)
     h->launches += 1;
     if ((e = launch_cg_update(B.ps, I.ue, st)) != cudaSuccess) return e;
     for (int k = 0; k < 4; ++k)
-        if ((e = (k == 0 || k == 2) ? hop_cg_plain(h, B.ps, k >= 2, I.k[k], st) : hop(h, B.ps, k >= 2, I.k[k], st)) !=
-            cudaSuccess)
-            return e;
+        if ((e = hop_cg(h, B.ps, k >= 2, I.k[k], st)) != cudaSuccess) return e;
     return cudaSuccess;
 }
 
@@ -937,6 +936,8 @@ int batch_impl(dwf_handle const *hs_in, const void *const *b4, void *const *x4, 
     CgScalars *hs_pinned = nullptr;
     CK(cudaMallocHost(&hs_pinned, sizeof(CgScalars) * (3 * (size_t)n + 4)));
     cudaStream_t cap = nullptr;
+    std::vector<cudaStream_t> branch;   // captured beside cap: one per further group
+    cudaEvent_t fork = nullptr;
     int worst = DWF_OK;
     int rc = DWF_OK;
     long long launches = 0;
@@ -949,6 +950,10 @@ int batch_impl(dwf_handle const *hs_in, const void *const *b4, void *const *x4, 
         A.base = nullptr;
         if (cap) cudaStreamDestroy(cap);
         cap = nullptr;
+        for (cudaStream_t b : branch) cudaStreamDestroy(b);
+        branch.clear();
+        if (fork) cudaEventDestroy(fork);
+        fork = nullptr;
         if (hs_pinned) cudaFreeHost(hs_pinned);
         hs_pinned = nullptr;
         if (skip_host) cudaFreeHost(skip_host);
@@ -1042,6 +1047,7 @@ int batch_impl(dwf_handle const *hs_in, const void *const *b4, void *const *x4, 
             CgUpdateArgs ue0;
             HopArgs k0[4];
             int ns = 0, sb = 0;
+            bool wa = false;   // every system on the FP32 default hop
         };
         std::vector<Group> groups(lsv.size());
         for (size_t g = 0; g < lsv.size(); ++g) {
@@ -1049,6 +1055,11 @@ int batch_impl(dwf_handle const *hs_in, const void *const *b4, void *const *x4, 
             for (int k = w.first; k < w.second; ++k)
                 if (runs[k].h->Ls == lsv[g]) G.mem.push_back(k);
             const int m = (int)G.mem.size();
+            G.wa = ps == DWF_F32;
+            for (int q = 0; q < m; ++q) {
+                const dwf_ctx *hq = runs[G.mem[q]].h;
+                G.wa = G.wa && (hq->hop_var[ps] < 0 || hq->hop_var[ps] == 9) && hq->mixmode[ps] < 2 && hq->sweep_zb[ps] <= 0;
+            }
             std::vector<CgUpdateArgs> ue(m);
             std::vector<HopArgs> kt[4];
             for (int q = 0; q < m; ++q) {
@@ -1063,25 +1074,28 @@ int batch_impl(dwf_handle const *hs_in, const void *const *b4, void *const *x4, 
                 I.ue.skip = skip_dev + (G.mem[q] - w.first);
                 ue[q] = I.ue;
                 for (int j = 0; j < 4; ++j) {
-                    HopArgs a = with_programs(R.h, ps, I.k[j]);
+                    HopArgs a = G.wa ? cg_programs(R.h, ps, I.k[j]) : with_programs(R.h, ps, I.k[j]);
                     a.skip = I.ue.skip;
                     kt[j].push_back(a);
                 }
             }
-            // one mixing mode per group (the kernels are compiled per mode); the
-            // dense matrices are always present, so disagreement falls back to them
-            int mixm = kt[0][0].mixmode;
-            for (int j = 0; j < 4; ++j)
-                for (int q = 0; q < m; ++q)
-                    if (kt[j][q].mixmode != mixm) mixm = 0;
-            for (int j = 0; j < 4; ++j)
-                for (int q = 0; q < m; ++q) kt[j][q].mixmode = mixm;
+            // one mixing mode per launch (the kernels are compiled per mode); the dense
+            // matrices are always present, so disagreement falls back to them
+            int mixm = ue[0].mixmode;
+            for (int q = 0; q < m; ++q)
+                if (ue[q].mixmode != mixm) mixm = 0;
             for (int q = 0; q < m; ++q) ue[q].mixmode = (mixm == 1) ? 1 : 0;
+            for (int j = 0; j < 4; ++j) {
+                int mj = kt[j][0].mixmode;
+                for (int q = 0; q < m; ++q)
+                    if (kt[j][q].mixmode != mj) mj = 0;
+                for (int q = 0; q < m; ++q) kt[j][q].mixmode = mj;
+            }
             G.ue0 = ue[0];
             for (int j = 0; j < 4; ++j) G.k0[j] = kt[j][0];
             dwf_ctx *hg = runs[G.mem[0]].h;
             G.ns = hg->hop_var[ps] == 0 ? hg->hop_ns[ps] : 0;
-            G.sb = hg->hop_var[ps] == 0 ? hg->hop_sb[ps] : 0;
+            G.sb = G.wa ? -1 : hg->hop_var[ps] == 0 ? hg->hop_sb[ps] : 0;
             G.ue = (CgUpdateArgs *)A.take(sizeof(CgUpdateArgs) * m);
             for (int j = 0; j < 4; ++j) G.k[j] = (HopArgs *)A.take(sizeof(HopArgs) * m);
             if (!G.ue || !G.k[3]) {
@@ -1092,32 +1106,42 @@ int batch_impl(dwf_handle const *hs_in, const void *const *b4, void *const *x4, 
             for (int j = 0; j < 4; ++j)
                 BCK(cudaMemcpyAsync(G.k[j], kt[j].data(), sizeof(HopArgs) * m, cudaMemcpyHostToDevice, st));
         }
-        auto launch_iteration = [&](cudaStream_t s2) -> cudaError_t {
+        auto launch_group = [&](Group &G, cudaStream_t s2) -> cudaError_t {
             cudaError_t e;
-            for (auto &G : groups) {
-                const int m = (int)G.mem.size();
-                if ((e = launch_cg_update_batch(ps, G.ue, m, G.ue0, s2)) != cudaSuccess) return e;
-                for (int j = 0; j < 4; ++j)
-                    if ((e = launch_hop_batch(ps, j >= 2, G.k[j], m, G.k0[j], G.ns, G.sb, s2)) != cudaSuccess)
-                        return e;
-            }
+            const int m = (int)G.mem.size();
+            if ((e = launch_cg_update_batch(ps, G.ue, m, G.ue0, s2)) != cudaSuccess) return e;
+            for (int j = 0; j < 4; ++j)
+                if ((e = launch_hop_batch(ps, j >= 2, G.k[j], m, G.k0[j], G.ns, G.sb, s2)) != cudaSuccess) return e;
             return cudaSuccess;
         };
         cudaGraphExec_t exec = nullptr;
         if (p->use_graph) {
             BCK(cudaStreamSynchronize(st));
+            // The groups share nothing: each is a branch of the graph, so that one's last CTAs
+            // and launch gaps are filled by the others'.
             cudaGraph_t g;
+            while (branch.size() + 1 < groups.size()) {
+                cudaStream_t b = nullptr;
+                BCK(cudaStreamCreateWithFlags(&b, cudaStreamNonBlocking));
+                branch.push_back(b);
+            }
+            if (!fork) BCK(cudaEventCreateWithFlags(&fork, cudaEventDisableTiming));
             BCK(cudaStreamBeginCapture(cap, cudaStreamCaptureModeThreadLocal));
-            for (int k = 0; k < N; ++k) {
-                cudaError_t e = launch_iteration(cap);
-                if (e != cudaSuccess) {
-                    cudaStreamEndCapture(cap, &g);
-                    cleanup();
-                    return dwf_cuda_error(e, "graph capture");
-                }
+            cudaError_t e = cudaEventRecord(fork, cap);
+            for (size_t g2 = 0; g2 < groups.size(); ++g2) {
+                cudaStream_t s2 = g2 ? branch[g2 - 1] : cap;
+                if (g2 && e == cudaSuccess) e = cudaStreamWaitEvent(s2, fork, 0);
+                for (int k = 0; k < N && e == cudaSuccess; ++k) e = launch_group(groups[g2], s2);
+            }
+            for (size_t g2 = 1; g2 < groups.size() && e == cudaSuccess; ++g2)
+                if ((e = cudaEventRecord(fork, branch[g2 - 1])) == cudaSuccess) e = cudaStreamWaitEvent(cap, fork, 0);
+            if (e != cudaSuccess) {
+                cudaStreamEndCapture(cap, &g);
+                cleanup();
+                return dwf_cuda_error(e, "graph capture");
             }
             BCK(cudaStreamEndCapture(cap, &g));
-            cudaError_t e = cudaGraphInstantiate(&exec, g, 0);
+            e = cudaGraphInstantiate(&exec, g, 0);
             cudaGraphDestroy(g);
             BCK(e);
         }
@@ -1137,7 +1161,8 @@ int batch_impl(dwf_handle const *hs_in, const void *const *b4, void *const *x4, 
                     BCK(e);
                 }
             } else {
-                for (int k = 0; k < N; ++k) BCK(launch_iteration(st));
+                for (int k = 0; k < N; ++k)
+                    for (auto &G : groups) BCK(launch_group(G, st));
             }
             launches += (long long)N * 5 * (long long)groups.size();
             for (int k = w.first; k < w.second; ++k)
@@ -1408,7 +1433,7 @@ int dwf_time_iteration(dwf_handle h, int prec, int reps, int flush_l2, double *u
         CK(launch_cg_update(prec, I.ue, st));
         CK(cudaEventRecord(ev[1], st));
         for (int k = 0; k < 4; ++k) {
-            CK((k == 0 || k == 2) ? hop_cg_plain(h, prec, k >= 2, I.k[k], st) : hop(h, prec, k >= 2, I.k[k], st));
+            CK(hop_cg(h, prec, k >= 2, I.k[k], st));
             CK(cudaEventRecord(ev[k + 2], st));
         }
         CK(cudaEventSynchronize(ev[5]));
