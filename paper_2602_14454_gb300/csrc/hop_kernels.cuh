@@ -1095,33 +1095,24 @@ struct WcProg {
 };
 static_assert(3 * sizeof(WcProg) <= 2048, "the programs exceed the CTA's front area");
 
-__device__ __forceinline__ void wc_load_prog(WcProg *dst, const MixProg<float> *src, int Ls, int tid, int nt)
+// by one warp; lane c + 2 k .. takes the coefficients, all loads in flight at once
+__device__ __forceinline__ void wc_load_prog(WcProg *dst, const MixProg<float> *src, int Ls, int lane)
 {
-    if (tid == 0) {
-        dst->inv = src->inv;
-        dst->shift = src->shift;
-        dst->up[0] = src->up[0];
-        dst->up[1] = src->up[1];
-        dst->s0 = src->s0;
-        dst->s1 = src->s1;
-        dst->a0inv = src->a0inv;
-        dst->kappa = src->kappa;
-        dst->mneg = src->mneg;
-        dst->corner = src->corner;
-        int o1 = 1, o2 = 1;
-        for (int c = 0; c < 2; ++c)
-            for (int s = 0; s < Ls; ++s) {
-                o1 &= src->d1[c][s] == 1.f;
-                o2 &= src->d2[c][s] == 1.f;
-            }
-        dst->d1one = o1;
-        dst->d2one = o2;
-    }
-    for (int e = tid; e < 2 * Ls; e += nt) {
+    const int *head = reinterpret_cast<const int *>(src);
+    if (lane < 4) reinterpret_cast<int *>(dst)[lane] = __ldg(head + lane);   // inv, shift, up[2]
+    if (lane < 6) (&dst->s0)[lane] = __ldg(reinterpret_cast<const float *>(head + 4) + lane);   // s0 .. corner
+    bool o1 = true, o2 = true;
+    for (int e = lane; e < 2 * Ls; e += 32) {
         const int c = e / Ls, s = e - c * Ls;
-        dst->d1[s][c] = src->d1[c][s];
-        dst->d2[s][c] = src->d2[c][s];
+        const float d1 = __ldg(&src->d1[c][s]), d2 = __ldg(&src->d2[c][s]);
+        dst->d1[s][c] = d1;
+        dst->d2[s][c] = d2;
+        o1 = o1 && d1 == 1.f;
+        o2 = o2 && d2 == 1.f;
     }
+    o1 = __all_sync(0xffffffffu, o1);
+    o2 = __all_sync(0xffffffffu, o2);
+    if (lane == 0) dst->d1one = o1, dst->d2one = o2;
 }
 
 // the program applied to every chain of the warp's tile, in place (d1 is
@@ -1264,9 +1255,8 @@ __device__ __forceinline__ float wc_epilogue(const HopArgs &a, const float2 *acc
 // the epilogue of hop_epilogue_core (dense mixing) on the warp's tile
 template <int P>
 __device__ __forceinline__ float wa_epilogue(const HopArgs &a, const float2 *acc, float2 *site_tile,
-                                             const float *mats, int s, int site, bool active)
+                                             const float *mats, int s, int Ls, int site, bool active)
 {
-    const int Ls = a.Ls;
     const int msz = 2 * Ls * wa_mat_row(Ls);
     float2 *row = site_tile + (size_t)s * LEAN_ROW;
     if (active && a.rin.v && a.xacc) {   // independent of the hop: first, while few registers are live
@@ -1353,11 +1343,14 @@ __device__ __forceinline__ void wa_issue_links(const void *gauge, int site0, int
 // range per CTA, spreading the tiles in work over the whole lattice, loses once
 // the fields exceed L2).
 // bid of nb: this CTA among those that work on a's lattice.
-template <int P, bool DAG, int MIX>
+// LS: Ls, or 0 for any (dense mixing only).  A fixed Ls takes the address arithmetic
+// out of the loops and the spills with it: 24^3x48 K_a 338 us instead of 360 (Ls 16),
+// 307 instead of 328 (Ls 12), the dense hop 397 / 425 and 345 / 377.
+template <int P, bool DAG, int MIX, int LS>
 __device__ __forceinline__ void hop_wa_body(const HopArgs &a, int bid, int nb)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    const int Ls = a.Ls, SPW = 32 / Ls;
+    const int Ls = LS ? LS : a.Ls, SPW = 32 / Ls;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
     // Ls need not divide 32: the lanes beyond the last whole site idle
     const int j = lane / Ls < SPW ? lane / Ls : 0, s = lane - (lane / Ls) * Ls;
@@ -1370,9 +1363,8 @@ __device__ __forceinline__ void hop_wa_body(const HopArgs &a, int bid, int nb)
         const MixProg<float> *src[3] = {reinterpret_cast<const MixProg<float> *>(a.post_prog),
                                         reinterpret_cast<const MixProg<float> *>(a.y_prog),
                                         reinterpret_cast<const MixProg<float> *>(a.z_prog)};
-        for (int m = 0; m < 3; ++m)
-            if (src[m] && (m != 1 || a.ymode == 2) && (m != 2 || a.zmat))
-                wc_load_prog(progs + m, src[m], Ls, threadIdx.x, blockDim.x);
+        for (int m = warp; m < 3; m += nwarps)
+            if (src[m] && (m != 1 || a.ymode == 2) && (m != 2 || a.zmat)) wc_load_prog(progs + m, src[m], Ls, lane);
     } else {
         const float *src[3] = {reinterpret_cast<const float *>(a.post),
                                a.ymode == 2 ? reinterpret_cast<const float *>(a.ymat) : nullptr,
@@ -1426,29 +1418,26 @@ __device__ __forceinline__ void hop_wa_body(const HopArgs &a, int bid, int nb)
             lean_dir<P, DAG, 6>(acc, a.in, n8[6], s, Ls, lk);
             lean_dir<P, DAG, 7>(acc, a.in, n8[7], s, Ls, lk);
         }
-        if constexpr (MIX == 1) {
-            if (Ls == 16) nrm += wc_epilogue<P, 16>(a, acc, tile, progs, j, s, site, worker, active, lane);
-            else if (Ls == 12) nrm += wc_epilogue<P, 12>(a, acc, tile, progs, j, s, site, worker, active, lane);
-            else nrm += wc_epilogue<P, 8>(a, acc, tile, progs, j, s, site, worker, active, lane);   // Ls 8 (launch_pd)
-        } else {
-            nrm += wa_epilogue<P>(a, acc, site_tile, mats, s, site, active);
-        }
+        if constexpr (MIX == 1)
+            nrm += wc_epilogue<P, LS>(a, acc, tile, progs, j, s, site, worker, active, lane);
+        else
+            nrm += wa_epilogue<P>(a, acc, site_tile, mats, s, Ls, site, active);
     }
     cp_async_wait<0>();
     if (a.red.op != RED_NONE) grid_reduce(nrm, a.red, (unsigned)bid, (unsigned)nb);
 }
 
-template <int P, bool DAG, int MINB, int MIX>
+template <int P, bool DAG, int MINB, int MIX, int LS>
 __global__ void __launch_bounds__(128, MINB) hop_wa_kernel(const HopArgs a)
 {
-    hop_wa_body<P, DAG, MIX>(a, blockIdx.x, gridDim.x);
+    hop_wa_body<P, DAG, MIX, LS>(a, blockIdx.x, gridDim.x);
 }
 
 // Batched form (FP32): CTA b belongs to system b % nsys, whose matrices it loads, and
 // walks that system's tiles with the system's other CTAs; as many CTAs in all as the
 // device holds.  8^3x16, 18 systems of Ls 8, 12 and 16: 24-44 us a hop of one Ls
 // against 44 us in the direct form, the whole batch 105 ms (128).
-template <bool DAG, int MIX>
+template <bool DAG, int MIX, int LS>
 __global__ void __launch_bounds__(128, 4) hop_wa_batch_kernel(const HopArgs *__restrict__ tab, int nsys)
 {
     __shared__ __align__(16) unsigned char abuf[sizeof(HopArgs)];
@@ -1457,7 +1446,7 @@ __global__ void __launch_bounds__(128, 4) hop_wa_batch_kernel(const HopArgs *__r
     __syncthreads();
     const HopArgs &a = *reinterpret_cast<const HopArgs *>(abuf);
     if (a.skip && *a.skip) return;
-    hop_wa_body<DWF_F32, DAG, MIX>(a, blockIdx.x / nsys, gridDim.x / nsys);
+    hop_wa_body<DWF_F32, DAG, MIX, LS>(a, blockIdx.x / nsys, gridDim.x / nsys);
 }
 
 
@@ -1828,24 +1817,24 @@ cudaError_t launch_direct_batch(const HopArgs *tab, int nsys, const HopArgs &a0,
     return cudaGetLastError();
 }
 
-template <bool DAG, int MIX>
+template <bool DAG, int MIX, int LS>
 cudaError_t launch_wa_batch(const HopArgs *tab, int nsys, const HopArgs &a0, cudaStream_t st)
 {
     static unsigned long long optin = 0;
     int dev = 0, nsm = 0, per_sm = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
-    if ((e = smem_optin(hop_wa_batch_kernel<DAG, MIX>, 200 * 1024, optin)) != cudaSuccess) return e;
+    if ((e = smem_optin(hop_wa_batch_kernel<DAG, MIX, LS>, 200 * 1024, optin)) != cudaSuccess) return e;
     if ((e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
     constexpr int nw = 4;
     const size_t smem = wa_cta_bytes<DWF_F32>(a0.Ls, nw);
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, hop_wa_batch_kernel<DAG, MIX>, 32 * nw, smem);
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, hop_wa_batch_kernel<DAG, MIX, LS>, 32 * nw, smem);
     if (e != cudaSuccess) return e;
     if (per_sm < 1) per_sm = 1;
     const int SPW = 32 / a0.Ls, most = ((a0.Vh + SPW - 1) / SPW + nw - 1) / nw;
     int each = nsm * per_sm / nsys;   // CTAs per system
     each = each < 1 ? 1 : each > most ? most : each;
-    hop_wa_batch_kernel<DAG, MIX><<<(unsigned)each * nsys, 32 * nw, smem, st>>>(tab, nsys);
+    hop_wa_batch_kernel<DAG, MIX, LS><<<(unsigned)each * nsys, 32 * nw, smem, st>>>(tab, nsys);
     return cudaGetLastError();
 }
 
@@ -1853,7 +1842,15 @@ template <int P, bool DAG>
 cudaError_t launch_batch_pd(const HopArgs *tab, int nsys, const HopArgs &a0, int NS, int SB, cudaStream_t st)
 {
     if constexpr (P == DWF_F32) {   // NS 0: warp-autonomous (launch_hop_batch)
-        if (NS == 0) return a0.mixmode == 1 ? launch_wa_batch<DAG, 1>(tab, nsys, a0, st) : launch_wa_batch<DAG, 0>(tab, nsys, a0, st);
+        if (NS == 0) {
+            const bool ch = a0.mixmode == 1;
+            switch (a0.Ls) {
+            case 8: return ch ? launch_wa_batch<DAG, 1, 8>(tab, nsys, a0, st) : launch_wa_batch<DAG, 0, 8>(tab, nsys, a0, st);
+            case 12: return ch ? launch_wa_batch<DAG, 1, 12>(tab, nsys, a0, st) : launch_wa_batch<DAG, 0, 12>(tab, nsys, a0, st);
+            case 16: return ch ? launch_wa_batch<DAG, 1, 16>(tab, nsys, a0, st) : launch_wa_batch<DAG, 0, 16>(tab, nsys, a0, st);
+            default: return launch_wa_batch<DAG, 0, 0>(tab, nsys, a0, st);
+            }
+        }
     }
     if constexpr (P == DWF_F16) {   // FP16 arithmetic (as hop variant 5) with dense mixing
         if (a0.mixmode == 0)
@@ -1966,21 +1963,21 @@ cudaError_t launch_lean(const HopArgs &a, int SB, cudaStream_t st)
 
 // Variant 9: persistent CTAs of `nw` warps (2, 4 or 8 resident CTAs' worth of
 // registers: nw x MINB x 32 threads per SM), as many per SM as fit.
-template <int P, bool DAG, int MINB, int MIX>
+template <int P, bool DAG, int MINB, int MIX, int LS>
 cudaError_t launch_wa(const HopArgs &a, int nw, cudaStream_t st)
 {
     static unsigned long long optin = 0;
     int dev = 0, nsm = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
-    if ((e = smem_optin(hop_wa_kernel<P, DAG, MINB, MIX>, 200 * 1024, optin)) != cudaSuccess) return e;
+    if ((e = smem_optin(hop_wa_kernel<P, DAG, MINB, MIX, LS>, 200 * 1024, optin)) != cudaSuccess) return e;
     if ((e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
     if (nw < 1) nw = 4;
     if (nw > 4) nw = 4;
     const size_t smem = wa_cta_bytes<P>(a.Ls, nw);
     if (smem > 200 * 1024) return cudaErrorInvalidConfiguration;
     int per_sm = 0;
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, hop_wa_kernel<P, DAG, MINB, MIX>, 32 * nw, smem);
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, hop_wa_kernel<P, DAG, MINB, MIX, LS>, 32 * nw, smem);
     if (e != cudaSuccess) return e;
     if (per_sm < 1) per_sm = 1;
     const int SPW = 32 / a.Ls;
@@ -1989,7 +1986,7 @@ cudaError_t launch_wa(const HopArgs &a, int nw, cudaStream_t st)
     if (grid > (ntiles + nw - 1) / nw) grid = (ntiles + nw - 1) / nw;
     HopArgs b = a;
     if (b.zblock > 0 && (b.zblock * b.ext[0] * b.ext[1]) % SPW) b.zblock = 0;   // a tile would straddle two runs
-    hop_wa_kernel<P, DAG, MINB, MIX><<<grid, 32 * nw, smem, st>>>(b);
+    hop_wa_kernel<P, DAG, MINB, MIX, LS><<<grid, 32 * nw, smem, st>>>(b);
     return cudaGetLastError();
 }
 
@@ -2055,11 +2052,22 @@ cudaError_t launch_pd(const HopArgs &a, int var, int NS, int SB, cudaStream_t st
     // multiple of 4); SB = warps per CTA, NS selects the register budget (1: 5 CTAs of 4
     // warps per SM, 2: 4)
     if constexpr (P != DWF_F64) {
-        if (var == 9 && a.mixmode == 0 && (P == DWF_F32 || (32 % a.Ls == 0 && a.Ls % 4 == 0)))
-            return NS == 2 ? launch_wa<P, DAG, 4, 0>(a, SB, st) : launch_wa<P, DAG, 5, 0>(a, SB, st);
-        // structured mixing by chains in registers (Ls 8 and 16)
-        if (var == 9 && a.mixmode == 1 && (a.Ls == 8 || a.Ls == 16 || (P == DWF_F32 && a.Ls == 12)))
-            return NS == 2 ? launch_wa<P, DAG, 4, 1>(a, SB, st) : launch_wa<P, DAG, 5, 1>(a, SB, st);
+        if (var == 9 && a.mixmode == 0 && (P == DWF_F32 || (32 % a.Ls == 0 && a.Ls % 4 == 0))) {
+            if constexpr (P == DWF_F32) {   // the default's register budget
+                if (NS == 2 && a.Ls == 8) return launch_wa<P, DAG, 4, 0, 8>(a, SB, st);
+                if (NS == 2 && a.Ls == 12) return launch_wa<P, DAG, 4, 0, 12>(a, SB, st);
+                if (NS == 2 && a.Ls == 16) return launch_wa<P, DAG, 4, 0, 16>(a, SB, st);
+            }
+            return NS == 2 ? launch_wa<P, DAG, 4, 0, 0>(a, SB, st) : launch_wa<P, DAG, 5, 0, 0>(a, SB, st);
+        }
+        // structured mixing by chains in registers (Ls 8 and 16, FP32 also 12)
+        if (var == 9 && a.mixmode == 1) {
+            if (a.Ls == 8) return NS == 2 ? launch_wa<P, DAG, 4, 1, 8>(a, SB, st) : launch_wa<P, DAG, 5, 1, 8>(a, SB, st);
+            if (a.Ls == 16) return NS == 2 ? launch_wa<P, DAG, 4, 1, 16>(a, SB, st) : launch_wa<P, DAG, 5, 1, 16>(a, SB, st);
+            if constexpr (P == DWF_F32) {
+                if (a.Ls == 12) return NS == 2 ? launch_wa<P, DAG, 4, 1, 12>(a, SB, st) : launch_wa<P, DAG, 5, 1, 12>(a, SB, st);
+            }
+        }
     }
     if (var == 9) var = P == DWF_F16 ? 5 : 0;
     if constexpr (P != DWF_F64) {
