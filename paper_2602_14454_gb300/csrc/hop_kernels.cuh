@@ -132,10 +132,9 @@ __device__ __forceinline__ void mix_into(const void *prog, const R *M, const Til
 // `bar` must call it.  Returns this thread's contribution to |o|^2.
 template <int P, int NS, int MIX = 0, typename T2, typename R, typename Bar>
 __device__ __forceinline__ R hop_epilogue_core(const HopArgs &a, T2 (*acc)[12], const TileCtx<T2> &tc,
-                                                    T2 *mytile, const R *mtx, int site, int x, int LsN, bool active,
-                                                    const Bar &bar)
+                                                    T2 *mytile, const R *mtx, int site, int x, int LsN, int Ls,
+                                                    bool active, const Bar &bar)
 {
-    const int Ls = a.Ls;
     const int msz = 2 * Ls * Ls;
     // tensor-core mixing: FP16 fields take the two-product form (its error is that of the FP16 storage)
     constexpr int MX = (MIX == 2 && P == DWF_F16) ? 3 : MIX;
@@ -258,7 +257,7 @@ __device__ __forceinline__ void hop_epilogue(const HopArgs &a, T2 (*acc)[12], T2
                                              int site, int x, int LsN, bool active)
 {
     const TileCtx<T2> tc = cta_tile(tile0, a.Ls);
-    const auto nrm = hop_epilogue_core<P, NS, MIX>(a, acc, tc, tile0 + j * tc.tstride, mtx, site, x, LsN, active,
+    const auto nrm = hop_epilogue_core<P, NS, MIX>(a, acc, tc, tile0 + j * tc.tstride, mtx, site, x, LsN, a.Ls, active,
                                                 CtaBarrier());
     if (a.red.op != RED_NONE) grid_reduce(nrm, a.red);
 }
@@ -410,14 +409,14 @@ __device__ __forceinline__ int sweep_site(const HopArgs &a, int p)
 // One tile of SB sites: blockDim = (Ls/NS, SB), site = u SB + threadIdx.y
 // (in the sweep order above when a tile never straddles a run of Bz A sites).
 // The norm reduction runs over the nb_red tiles that share a.red.
-template <int P, bool DAG, int NS, int MIX, bool H2 = false>
+template <int P, bool DAG, int NS, int MIX, bool H2 = false, int LS = 0>
 __device__ __forceinline__ void hop_direct_tile(const HopArgs &a, int u, unsigned nb_red)
 {
     typedef typename Tr<P>::real R;
     typedef typename Tr<P>::pair T2;
     typedef typename Tr<P>::link_t link_t;
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    const int Ls = a.Ls;
+    const int Ls = LS ? LS : a.Ls;
     const int LsN = Ls / NS;
     const int x = threadIdx.x;
     const int j = threadIdx.y;
@@ -443,7 +442,7 @@ __device__ __forceinline__ void hop_direct_tile(const HopArgs &a, int u, unsigne
         gather8<P, DAG, NS, H2>(acc, a, n8, x, LsN, Ls, U);
     }
     const TileCtx<T2> tc = cta_tile(tile, Ls);
-    const auto nrm = hop_epilogue_core<P, NS, MIX>(a, acc, tc, tile + j * tc.tstride, mtx, site, x, LsN, active,
+    const auto nrm = hop_epilogue_core<P, NS, MIX>(a, acc, tc, tile + j * tc.tstride, mtx, site, x, LsN, Ls, active,
                                                      CtaBarrier());
     if (a.red.op != RED_NONE) grid_reduce(nrm, a.red, u, nb_red);
 }
@@ -459,10 +458,10 @@ __global__ void __launch_bounds__(256) hop_kernel(const HopArgs a)
 // 64 registers (FP16: 8 CTAs of 128 threads per SM) the hop at 16^3x32, Ls 16
 // went from 96.2 us to 85.8 us, capped at 85 (FP32: 6 CTAs) from 117.8 us to
 // 106.3 us.
-template <int P, bool DAG, int MIX, bool H2>
+template <int P, bool DAG, int MIX, bool H2, int LS>
 __global__ void __launch_bounds__(256, P == DWF_F16 ? 4 : 3) hop_kernel_occ(const HopArgs a)
 {
-    hop_direct_tile<P, DAG, 1, MIX, H2>(a, blockIdx.x, gridDim.x);
+    hop_direct_tile<P, DAG, 1, MIX, H2, LS>(a, blockIdx.x, gridDim.x);
 }
 
 // Batched form: one launch over nsys systems that share Ls and the CTA shape
@@ -609,7 +608,7 @@ __global__ void __launch_bounds__(256) hop_sweep_kernel(const HopArgs a, int tpc
             hop_dir<P, DAG, 7, NS>(acc, a.in, n8[7], x, LsN, Ls, U);
         }
         __syncthreads();   // the previous tile's epilogue is done with `tile`
-        nrm += hop_epilogue_core<P, NS>(a, acc, cta_tile(tile, Ls), tile + j * tstride, mtx, site, x, LsN, active,
+        nrm += hop_epilogue_core<P, NS>(a, acc, cta_tile(tile, Ls), tile + j * tstride, mtx, site, x, LsN, Ls, active,
                                         CtaBarrier());
     }
     if (a.red.op != RED_NONE) grid_reduce(nrm, a.red);
@@ -1773,15 +1772,26 @@ size_t direct_smem(int Ls, int SB)
     return (size_t)SB * (Ls * 12 + 2) * sizeof(T2) + (size_t)3 * 2 * Ls * Ls * sizeof(R);
 }
 
+template <int P, bool DAG, int MIX, bool H2, int LS>
+cudaError_t launch_direct_occ(const HopArgs &a, int SB, cudaStream_t st)
+{
+    static unsigned long long optin = 0;
+    cudaError_t e = smem_optin(hop_kernel_occ<P, DAG, MIX, H2, LS>, 200 * 1024, optin);
+    if (e != cudaSuccess) return e;
+    hop_kernel_occ<P, DAG, MIX, H2, LS><<<(a.Vh + SB - 1) / SB, dim3(a.Ls, SB), direct_smem<P>(a.Ls, SB), st>>>(a);
+    return cudaGetLastError();
+}
+
 template <int P, bool DAG, int NS, int MIX = 0, bool H2 = false>
 cudaError_t launch_direct(const HopArgs &a, int SB, cudaStream_t st)
 {
     if constexpr (NS == 1 && MIX == 0 && ((P == DWF_F16 && H2) || (P == DWF_F32 && !H2))) {
-        static unsigned long long optin_occ = 0;
-        cudaError_t e = smem_optin(hop_kernel_occ<P, DAG, MIX, H2>, 200 * 1024, optin_occ);
-        if (e != cudaSuccess) return e;
-        hop_kernel_occ<P, DAG, MIX, H2><<<(a.Vh + SB - 1) / SB, dim3(a.Ls, SB), direct_smem<P>(a.Ls, SB), st>>>(a);
-        return cudaGetLastError();
+        if constexpr (P == DWF_F16) {
+            if (a.Ls == 8) return launch_direct_occ<P, DAG, MIX, H2, 8>(a, SB, st);
+            if (a.Ls == 12) return launch_direct_occ<P, DAG, MIX, H2, 12>(a, SB, st);
+            if (a.Ls == 16) return launch_direct_occ<P, DAG, MIX, H2, 16>(a, SB, st);
+        }
+        return launch_direct_occ<P, DAG, MIX, H2, 0>(a, SB, st);
     }
     static unsigned long long optin = 0;
     {
