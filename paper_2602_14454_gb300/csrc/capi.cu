@@ -297,8 +297,16 @@ HopArgs cg_programs(dwf_ctx *h, int prec, const HopArgs &a)
 cudaError_t hop_cg(dwf_ctx *h, int prec, bool dag, const HopArgs &a, cudaStream_t st)
 {
     if (prec == DWF_F64) return hop(h, prec, dag, a, st);
+    const HopArgs c = cg_programs(h, prec, a);
+    int var = h->hop_var[prec];
+    // FP16's default is the direct variant 5, but K_d (two banded mixings) is faster
+    // warp-autonomous at Ls 8 and 16: 51 / 61 us and 90 / 114 us at 16^3x32, 213 / 259 and
+    // 428 / 508 us at 24^3x48 (the dense K_a and K_b are not: 82 / 82, 418 / 365 us at Ls 16)
+    if (prec == DWF_F16 && var < 0 && c.mixmode == 0 && (h->Ls == 8 || h->Ls == 16) && c.post_band && c.ymode == 2 &&
+        c.y_band && !c.zmat && h->hop_ns[prec] == 0 && h->hop_sb[prec] == 0)
+        var = 9;
     h->launches += 1;
-    return launch_hop(prec, dag, cg_programs(h, prec, a), h->hop_var[prec], h->hop_ns[prec], h->hop_sb[prec], st);
+    return launch_hop(prec, dag, c, var, h->hop_ns[prec], h->hop_sb[prec], st);
 }
 
 // A field that only hops and mixings read: FP64 fields are kept as blocks then.

@@ -2063,10 +2063,11 @@ cudaError_t launch_pd(const HopArgs &a, int var, int NS, int SB, cudaStream_t st
     // warps per SM, 2: 4)
     if constexpr (P != DWF_F64) {
         if (var == 9 && a.mixmode == 0 && (P == DWF_F32 || (32 % a.Ls == 0 && a.Ls % 4 == 0))) {
-            if constexpr (P == DWF_F32) {   // the default's register budget
-                if (NS == 2 && a.Ls == 8) return launch_wa<P, DAG, 4, 0, 8>(a, SB, st);
+            // the default's register budget
+            if (NS == 2 && a.Ls == 8) return launch_wa<P, DAG, 4, 0, 8>(a, SB, st);
+            if (NS == 2 && a.Ls == 16) return launch_wa<P, DAG, 4, 0, 16>(a, SB, st);
+            if constexpr (P == DWF_F32) {
                 if (NS == 2 && a.Ls == 12) return launch_wa<P, DAG, 4, 0, 12>(a, SB, st);
-                if (NS == 2 && a.Ls == 16) return launch_wa<P, DAG, 4, 0, 16>(a, SB, st);
             }
             return NS == 2 ? launch_wa<P, DAG, 4, 0, 0>(a, SB, st) : launch_wa<P, DAG, 5, 0, 0>(a, SB, st);
         }
