@@ -271,21 +271,14 @@ void source_diagonal(const dwf_ctx *h, double y[2])
     y[1] = m[(size_t)h->Ls * h->Ls - 1];
 }
 
-cudaError_t hop(dwf_ctx *h, int prec, bool dag, const HopArgs &a, cudaStream_t st)
-{
-    if (prec == DWF_F64 && h->use_fx()) return hop_fx(h, dag, a, st);
-    h->launches += 1;
-    return launch_hop(prec, dag, with_programs(h, prec, a), h->hop_var[prec], h->hop_ns[prec], h->hop_sb[prec], st);
-}
-
-// A hop of the CG iteration.  In FP32, when the caller left the mixing mode and the
-// hop variant at their defaults, the hops that mix with inverses only (K_a, K_b, K_c)
-// take the structured mixing by register chains at Ls 12 and 16: it reads every tile
+// The programs of a hop.  In FP32, when the caller left the mixing mode and the hop
+// variant at their defaults, the hops that mix with inverses only (K_a, K_b, K_c of the
+// CG iteration) take the structured mixing by register chains at Ls 12 and 16: it reads every tile
 // element once where the dense form reads the site's tile and a matrix row per
 // output.  24^3x48, chains against dense: Ls 16 K_a 372 / 426 us, K_b 533 / 591 us;
 // Ls 12 338 / 380, 472 / 515; at Ls 8 the dense form wins (K_a 190 / 186, K_b
 // 261 / 240).  The banded K_d reads three rows per output and stays dense (449 / 578).
-HopArgs cg_programs(dwf_ctx *h, int prec, const HopArgs &a)
+HopArgs hop_programs(dwf_ctx *h, int prec, const HopArgs &a)
 {
     if (prec == DWF_F32 && h->mixmode[prec] < 0 && h->fm.structured && (h->Ls == 12 || h->Ls == 16) &&
         (h->hop_var[prec] < 0 || h->hop_var[prec] == 9) && a.ymode != 2 && !a.rin.v) {
@@ -294,10 +287,10 @@ HopArgs cg_programs(dwf_ctx *h, int prec, const HopArgs &a)
     }
     return with_programs(h, prec, a);
 }
-cudaError_t hop_cg(dwf_ctx *h, int prec, bool dag, const HopArgs &a, cudaStream_t st)
+cudaError_t hop(dwf_ctx *h, int prec, bool dag, const HopArgs &a, cudaStream_t st)
 {
-    if (prec == DWF_F64) return hop(h, prec, dag, a, st);
-    const HopArgs c = cg_programs(h, prec, a);
+    if (prec == DWF_F64 && h->use_fx()) return hop_fx(h, dag, a, st);
+    const HopArgs c = hop_programs(h, prec, a);
     int var = h->hop_var[prec];
     // FP16's default is the direct variant 5, but K_d (two banded mixings) is faster
     // warp-autonomous at Ls 8 and 16: 51 / 61 us and 90 / 114 us at 16^3x32, 213 / 259 and
@@ -539,6 +532,8 @@ static int create_impl(const int dims[4], int Ls, double M0, double mf, const do
             d.s0 = s.s0, d.s1 = s.s1, d.a0inv = s.a0inv, d.kappa = s.kappa, d.mneg = s.mneg, d.corner = s.corner;
             f.s0 = (float)s.s0, f.s1 = (float)s.s1, f.a0inv = (float)s.a0inv, f.kappa = (float)s.kappa;
             f.mneg = (float)s.mneg, f.corner = (float)s.corner;
+            d.c1 = s.s0 * s.a0inv, d.c2 = s.s0 * s.kappa + s.s1;
+            f.c1 = (float)d.c1, f.c2 = (float)d.c2;
         }
         if ((e = cudaMalloc(&h->progs_dev[0], pd.size() * sizeof(pd[0]))) != cudaSuccess) return fail(e, "cudaMalloc");
         if ((e = cudaMalloc(&h->progs_dev[1], pf.size() * sizeof(pf[0]))) != cudaSuccess) return fail(e, "cudaMalloc");
@@ -1218,7 +1213,7 @@ int dwf_autotune(dwf_handle h, int prec, const char *cache_path, void *stream)
     }
     double best = 1e30;
     int bvar = -1, bns = 0, bsb = 0, bmix = 0;
-    if (prec == DWF_F64) {   // the fixed-point hop, the default, has no variant number or mixing mode of its own
+    {   // the defaults, which choose by operation: FP64 blocks, chains or rows
         h->mixmode[prec] = h->hop_var[prec] = bmix = -1;
         h->hop_ns[prec] = h->hop_sb[prec] = 0;
         double by = 0;

@@ -274,6 +274,7 @@ template <typename R>
 struct MixProg {
     int inv, shift, up[2];
     R s0, s1, a0inv, kappa, mneg, corner;
+    R c1, c2;   // inv and shift in one step: c1 v_s + c2 x_{s-1}, c1 = s0 / alpha0, c2 = s0 kappa + s1
     R d1[2][LS_MAX], d2[2][LS_MAX];
 };
 

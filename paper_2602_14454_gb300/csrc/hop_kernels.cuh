@@ -1089,7 +1089,7 @@ __host__ __device__ constexpr int wc_site_stride(int Ls) { return Ls * 14 + (28 
 // a program in shared memory with the chirality-interleaved d vectors
 struct WcProg {
     int inv, shift, up[2], d1one, d2one;
-    float s0, s1, a0inv, kappa, mneg, corner;
+    float s0, s1, a0inv, kappa, mneg, corner, c1, c2;
     float d1[LS_MAX][2], d2[LS_MAX][2];
 };
 static_assert(3 * sizeof(WcProg) <= 2048, "the programs exceed the CTA's front area");
@@ -1099,7 +1099,7 @@ __device__ __forceinline__ void wc_load_prog(WcProg *dst, const MixProg<float> *
 {
     const int *head = reinterpret_cast<const int *>(src);
     if (lane < 4) reinterpret_cast<int *>(dst)[lane] = __ldg(head + lane);   // inv, shift, up[2]
-    if (lane < 6) (&dst->s0)[lane] = __ldg(reinterpret_cast<const float *>(head + 4) + lane);   // s0 .. corner
+    if (lane < 8) (&dst->s0)[lane] = __ldg(reinterpret_cast<const float *>(head + 4) + lane);   // s0 .. c2
     bool o1 = true, o2 = true;
     for (int e = lane; e < 2 * Ls; e += 32) {
         const int c = e / Ls, s = e - c * Ls;
@@ -1124,7 +1124,6 @@ __device__ __forceinline__ void wc_chains(const WcProg *pg, float *tile, int lan
     const int chi = (lane >> 1) & 1;
     const bool up = pg->up[chi] != 0;
     const bool o1 = pg->d1one != 0, o2 = pg->d2one != 0;
-    const float kappa = pg->kappa, a0inv = pg->a0inv, mneg = pg->mneg, s0 = pg->s0, s1 = pg->s1;
 #pragma unroll 1
     for (int c = lane; c < NCH; c += 32) {
         const int jj = c / 24, k = c - jj * 24;
@@ -1137,27 +1136,32 @@ __device__ __forceinline__ void wc_chains(const WcProg *pg, float *tile, int lan
             if (!o1) v[u] *= pg->d1[sl][chi];
         }
         if (pg->inv) {
+            const float kappa = pg->kappa, a0inv = pg->a0inv;
             float acc = 0.f;
 #pragma unroll
             for (int u = 0; u < LS; ++u) acc = fmaf(kappa, acc, v[u]);
-            float prev = mneg * (acc * a0inv * pg->corner);
-#pragma unroll
-            for (int u = 0; u < LS; ++u) {
-                const float w = fmaf(v[u], a0inv, kappa * prev);
-                prev = w;
-                v[u] = w;
-            }
+            float prev = pg->mneg * (acc * a0inv * pg->corner);   // -m x_last: what both the recurrence and the shift start from
             if (pg->shift) {
-                float prevs = mneg * v[LS - 1];
+                // the shifted output from v and x_{u-1}: one pass, and x_u's roundings stay out of it (error
+                // of the even-odd application against 64 bits, b 1.5 c 0.5: 7.3e-8; from x_u and x_{u-1}
+                // 7.9e-8, the dense form 7.6e-8)
+                const float c1 = pg->c1, c2 = pg->c2;
 #pragma unroll
                 for (int u = 0; u < LS; ++u) {
-                    const float tt = v[u];
-                    v[u] = fmaf(s0, tt, s1 * prevs);
-                    prevs = tt;
+                    const float t = v[u];
+                    v[u] = fmaf(c1, t, c2 * prev);
+                    prev = fmaf(t, a0inv, kappa * prev);
+                }
+            } else {
+#pragma unroll
+                for (int u = 0; u < LS; ++u) {
+                    prev = fmaf(v[u], a0inv, kappa * prev);
+                    v[u] = prev;
                 }
             }
         } else if (pg->shift) {
-            float prevs = mneg * v[LS - 1];
+            const float s0 = pg->s0, s1 = pg->s1;
+            float prevs = pg->mneg * v[LS - 1];
 #pragma unroll
             for (int u = 0; u < LS; ++u) {
                 const float tt = v[u];

@@ -34,9 +34,8 @@ using namespace dwf;
 namespace dwf_detail {
 HopArgs hop_args(dwf_ctx *h, int prec, int out_par, FieldRef in, FieldRef out, int post);
 HopArgs with_programs(dwf_ctx *h, int prec, const HopArgs &a0);
-HopArgs cg_programs(dwf_ctx *h, int prec, const HopArgs &a);
+HopArgs hop_programs(dwf_ctx *h, int prec, const HopArgs &a);
 cudaError_t hop(dwf_ctx *h, int prec, bool dag, const HopArgs &a, cudaStream_t st);
-cudaError_t hop_cg(dwf_ctx *h, int prec, bool dag, const HopArgs &a, cudaStream_t st);
 size_t source_scratch_bytes(const dwf_ctx *h);
 cudaError_t source_hops(dwf_ctx *h, const void *b4, void *scratch, FieldRef hop2[2], cudaStream_t st);
 void source_diagonal(const dwf_ctx *h, double y[2]);
@@ -182,7 +181,7 @@ cudaError_t inner_iteration(dwf_ctx *h, const Bufs &B, cudaStream_t st)
     h->launches += 1;
     if ((e = launch_cg_update(B.ps, I.ue, st)) != cudaSuccess) return e;
     for (int k = 0; k < 4; ++k)
-        if ((e = hop_cg(h, B.ps, k >= 2, I.k[k], st)) != cudaSuccess) return e;
+        if ((e = hop(h, B.ps, k >= 2, I.k[k], st)) != cudaSuccess) return e;
     return cudaSuccess;
 }
 
@@ -1074,7 +1073,7 @@ int batch_impl(dwf_handle const *hs_in, const void *const *b4, void *const *x4, 
                 I.ue.skip = skip_dev + (G.mem[q] - w.first);
                 ue[q] = I.ue;
                 for (int j = 0; j < 4; ++j) {
-                    HopArgs a = G.wa ? cg_programs(R.h, ps, I.k[j]) : with_programs(R.h, ps, I.k[j]);
+                    HopArgs a = G.wa ? hop_programs(R.h, ps, I.k[j]) : with_programs(R.h, ps, I.k[j]);
                     a.skip = I.ue.skip;
                     kt[j].push_back(a);
                 }
@@ -1433,7 +1432,7 @@ int dwf_time_iteration(dwf_handle h, int prec, int reps, int flush_l2, double *u
         CK(launch_cg_update(prec, I.ue, st));
         CK(cudaEventRecord(ev[1], st));
         for (int k = 0; k < 4; ++k) {
-            CK(hop_cg(h, prec, k >= 2, I.k[k], st));
+            CK(hop(h, prec, k >= 2, I.k[k], st));
             CK(cudaEventRecord(ev[k + 2], st));
         }
         CK(cudaEventSynchronize(ev[5]));
