@@ -111,8 +111,8 @@ const char *dwf_last_error(void);
 
 /* Copy the links U_mu(x) of the 4D Wilson kernel, eq. (Wilson_matrix)
  * (device, layout above, SU(3) expected but not checked) into the handle: the
- * boundary phases are folded in and an internal copy in FP64, FP32 and FP16
- * is made for each output parity; the caller's buffer is not kept.  Must be
+ * boundary phases are folded in and an internal copy in FP64, FP32, FP16 and
+ * fixed point is made for each output parity; the caller's buffer is not kept.  Must be
  * called before any operator call; calling it again replaces the links.
  * Errors: DWF_EINVAL (NULL handle or U, U not 16-byte aligned), DWF_ECUDA. */
 int dwf_set_gauge(dwf_handle h, const void *U, void *stream);

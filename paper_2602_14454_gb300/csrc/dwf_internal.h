@@ -120,6 +120,8 @@ struct HopArgs {
     int post_band = 0, y_band = 0, z_band = 0;   // the matrix is cyclic tridiagonal (dense mode reads 3 per row)
     // fixed-point FP64 hop: the matrices' constants (mats_fx), with *_band 2 for a diagonal matrix
     const int4 *post_fx = nullptr, *y_fx = nullptr, *z_fx = nullptr;
+    const int4 *gauge_fx = nullptr;    // the links as limbs, [Vh][8][9], and their exponents [Vh][8]
+    const int *gauge_e = nullptr;
     int zblock = 0;                // sweep the lattice in columns of zblock z-planes (0: index order)
 };
 
@@ -221,7 +223,9 @@ cudaError_t launch_zero(int prec, FieldRef f, int Vh, int Ls, cudaStream_t st);
 // gauge and index tables
 cudaError_t launch_build_tables(const int dims[4], int *nbr, int *eo2lex, cudaStream_t st);
 cudaError_t launch_pack_gauge(const double *U, const int dims[4], const int bc[4], void *g64, void *g32, void *g16,
-                              cudaStream_t st);
+                              int4 *gfx, int *ge, cudaStream_t st);
+// limbs and exponents of n links from their FP64 copy
+cudaError_t launch_links_to_limbs(const void *g64, int4 *gfx, int *ge, size_t n, cudaStream_t st);
 
 // projection on canonical 5D fields (FP64)
 cudaError_t launch_project4d(const double *x5, double *x4, int V, int Ls, cudaStream_t st);
@@ -317,6 +321,8 @@ struct dwf_ctx {
     int *nbr = nullptr;       // [2][Vh][8]
     int *eo2lex = nullptr;    // [2][Vh]
     void *gauge[3] = {nullptr, nullptr, nullptr};      // per precision, [2][Vh][8][18]
+    int4 *gauge_fx = nullptr;   // the links as fixed-point limbs, [2][Vh][8][9], and exponents, [2][Vh][8]
+    int *gauge_e = nullptr;
     bool has_gauge = false;
     double *partials = nullptr;
     unsigned *counter = nullptr;

@@ -2,9 +2,10 @@
 // operator.  Same launch, arguments and epilogue as the hop of hop_kernels.cuh;
 // the input field is a block field, y and the output FP64 or block fields, rin FP64.
 //
-// A CTA takes SB sites x all Ls slices, one (site, s) per thread.  It copies its
-// sites' links (FP64) to shared memory and turns them into limbs there, once for
-// all slices.  The threads walk the eight directions in one loop (unrolled, its code
+// A CTA takes SB sites x all Ls slices, one (site, s) per thread.  Its sites' links
+// come to shared memory as limbs, made when the links are set (turning FP64 links into
+// limbs here cost 2 % at Ls 16, 8 % at Ls 10 and half of the two-slice source: 1632
+// against 725 us at 24^3x48).  The threads walk the eight directions in one loop (unrolled, its code
 // no longer fits the instruction cache): each has its neighbour's block copied
 // asynchronously into its own shared slots one direction ahead, projects, multiplies
 // and reconstructs in integers.  The eight directions' exponents are known before
@@ -28,6 +29,7 @@ namespace {
 // 2^(e - 59) for H and 2^(eu - 59) for U, Q comes in 2^(e + eu - 56); the sums of the
 // cross products stay below 2^62.6 and are rounded at 2^31, eight directions' Q below
 // 2^62.6.
+template <bool GLOBAL>
 __device__ __forceinline__ void fx_su3(const int4 *u, const longlong2 *Hx, const longlong2 *Hy, int sh, longlong2 *Qx,
                                        longlong2 *Qy)
 {
@@ -46,7 +48,7 @@ __device__ __forceinline__ void fx_su3(const int4 *u, const longlong2 *Hx, const
         for (int p = 0; p < 2; ++p) rh[p] = ih[p] = 0, rx[p] = ix[p] = 1 << 30;
 #pragma unroll
         for (int b = 0; b < 3; ++b) {
-            const int4 q = u[a * 3 + b];
+            const int4 q = GLOBAL ? __ldg(u + a * 3 + b) : u[a * 3 + b];
 #pragma unroll
             for (int p = 0; p < 2; ++p) {
                 fx_mad(xl[b][p], xh[b][p], q.x, q.y, rh[p], rx[p]);
@@ -139,38 +141,13 @@ struct FxSmem {
     int *nb;      // [SB][8] neighbours
     int *te;      // [SB][Ls]
 };
+// two slices (the 5D source) read their links from global memory: with two threads to
+// a site, staging them would only cost occupancy
+__host__ __device__ constexpr bool fx_global_links(int Ls) { return Ls == 2; }
 __host__ __device__ inline size_t fx_smem_bytes(int Ls, int SB)
 {
-    return (size_t)SB * (72 + fx_site_stride(Ls)) * sizeof(int4) + (size_t)SB * (16 + Ls) * sizeof(int);
-}
-
-// The links of sites site0 .. site0 + n - 1 as limbs and exponents.  A link's entry
-// is U 2^(eu - 59).
-__device__ __forceinline__ void fx_stage_links(const double *gauge, int site0, int n, const FxSmem &sm, int tid, int nt)
-{
-    const double2 *src = reinterpret_cast<const double2 *>(gauge) + (size_t)site0 * 72;
-    double2 *d = reinterpret_cast<double2 *>(sm.u);
-    for (int i = tid; i < n * 72; i += nt) d[i] = __ldg(src + i);
-    __syncthreads();
-    for (int l = tid; l < n * 8; l += nt) {
-        uint32_t m = 0, low = 0;
-#pragma unroll
-        for (int k = 0; k < 9; ++k) {
-            const double2 q = d[l * 9 + k];
-            m = max(m, max((uint32_t)__double2hiint(q.x) & 0x7fffffffu, (uint32_t)__double2hiint(q.y) & 0x7fffffffu));
-            low |= (uint32_t)__double2loint(q.x) | (uint32_t)__double2loint(q.y);
-        }
-        sm.eu[l] = fx_exponent(m, low);
-    }
-    __syncthreads();
-    for (int i = tid; i < n * 72; i += nt) {
-        const double2 q = d[i];
-        const int e = sm.eu[i / 9];
-        int4 w;
-        fx_limbs31s(fx_from_double(q.x, e, FX_BITS), w.x, w.y);
-        fx_limbs31s(fx_from_double(q.y, e, FX_BITS), w.z, w.w);
-        sm.u[i] = w;
-    }
+    return (size_t)SB * ((fx_global_links(Ls) ? 0 : 72) + fx_site_stride(Ls)) * sizeof(int4) +
+           (size_t)SB * (16 + Ls) * sizeof(int);
 }
 
 // LS: Ls, or 0 for any (the fixed ones save the address arithmetic)
@@ -178,13 +155,14 @@ template <bool DAG, int LS>
 __global__ void __launch_bounds__(128, 4) hop_fx_kernel(const HopArgs a)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    const int Ls = LS ? LS : a.Ls, SB = LS ? 128 / LS : blockDim.y, s = threadIdx.x, j = threadIdx.y;
+    const int Ls = LS ? LS : a.Ls, SB = LS ? 128 / LS : (int)blockDim.y, s = threadIdx.x, j = threadIdx.y;
     const int tid = j * Ls + s, nt = Ls * SB, B = fx_mix_bits(Ls);
     const int site0 = blockIdx.x * SB, site = site0 + j;
     const bool active = site < a.Vh;
     FxSmem sm;
+    constexpr bool GL = fx_global_links(LS);
     sm.u = reinterpret_cast<int4 *>(smem_raw);
-    sm.tile = sm.u + SB * 72;
+    sm.tile = sm.u + (GL ? 0 : SB * 72);
     sm.eu = reinterpret_cast<int *>(sm.tile + SB * fx_site_stride(Ls));
     sm.nb = sm.eu + SB * 8;
     sm.te = sm.nb + SB * 8;
@@ -192,14 +170,30 @@ __global__ void __launch_bounds__(128, 4) hop_fx_kernel(const HopArgs a)
     int *te = sm.te + j * Ls;
     const int *nb = sm.nb + j * 8;
 
-    for (int i = tid; i < min(SB, a.Vh - site0) * 8; i += nt) sm.nb[i] = __ldg(a.nbr + (size_t)site0 * 8 + i);
-    __syncthreads();
-    if (active) fx_fetch(slot, nt, a.in, nb[0], s, Ls);
+    const int nsites = min(SB, a.Vh - site0);
+    if (!GL) {
+        const int4 *src = a.gauge_fx + (size_t)site0 * 72;
+        const uint32_t d = (uint32_t)__cvta_generic_to_shared(sm.u);
+        for (int i = tid; i < nsites * 72; i += nt)
+            asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(d + i * 16), "l"(src + i) : "memory");
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    }
+    for (int i = tid; i < nsites * 8; i += nt) {
+        sm.nb[i] = __ldg(a.nbr + (size_t)site0 * 8 + i);
+        sm.eu[i] = __ldg(a.gauge_e + (size_t)site0 * 8 + i);
+    }
     int e8[8];
-    if (active)
+    if (active) {
+        const int4 *p = reinterpret_cast<const int4 *>(a.nbr + (size_t)site * 8);
+        const int4 q0 = __ldg(p), q1 = __ldg(p + 1);
+        fx_fetch(slot, nt, a.in, q0.x, s, Ls);
+        const int n8[8] = {q0.x, q0.y, q0.z, q0.w, q1.x, q1.y, q1.z, q1.w};
 #pragma unroll
-        for (int d = 0; d < 8; ++d) e8[d] = __ldg(a.in.fx + (size_t)nb[d] * Ls + s);
-    fx_stage_links(reinterpret_cast<const double *>(a.gauge), site0, min(SB, a.Vh - site0), sm, tid, nt);
+        for (int d = 0; d < 8; ++d) e8[d] = __ldg(a.in.fx + (size_t)n8[d] * Ls + s);
+    } else {
+        asm volatile("cp.async.commit_group;" ::: "memory");   // the same number of groups as the others
+    }
+    asm volatile("cp.async.wait_group 1;" ::: "memory");   // the links; the first block may still be on its way
     __syncthreads();
 
     longlong2 acc[12];
@@ -217,7 +211,7 @@ __global__ void __launch_bounds__(128, 4) hop_fx_kernel(const HopArgs a)
         uint64_t shifts = 0;   // emax - e per direction, at most 63, eight bits each
 #pragma unroll
         for (int d = 0; d < 8; ++d) shifts |= (uint64_t)(uint32_t)min(emax - e8[d], 63) << (8 * d);
-        const int4 *u = sm.u + j * 72;
+        const int4 *u = GL ? a.gauge_fx + (size_t)site * 72 : sm.u + j * 72;
 #pragma unroll 1
         for (int d = 0; d < 8; ++d) {
             longlong2 Hx[3], Hy[3], Qx[3], Qy[3];
@@ -229,7 +223,7 @@ __global__ void __launch_bounds__(128, 4) hop_fx_kernel(const HopArgs a)
                 fx_project<DAG>(d, v, Hx, Hy);
             }
             if (d < 7) fx_fetch(slot, nt, a.in, nb[d + 1], s, Ls);   // into the same slots: this block is in registers
-            fx_su3(u + d * 9, Hx, Hy, (int)(shifts >> (8 * d)) & 63, Qx, Qy);
+            fx_su3<GL>(u + d * 9, Hx, Hy, (int)(shifts >> (8 * d)) & 63, Qx, Qy);
             fx_reconstruct<DAG>(d, acc, Qx, Qy);
         }
     }
@@ -347,6 +341,7 @@ template <bool DAG>
 cudaError_t hop_fx_launch(const HopArgs &a, cudaStream_t st)
 {
     switch (a.Ls) {
+    case 2: return hop_fx_launch_ls<DAG, 2>(a, st);
     case 8: return hop_fx_launch_ls<DAG, 8>(a, st);
     case 12: return hop_fx_launch_ls<DAG, 12>(a, st);
     case 16: return hop_fx_launch_ls<DAG, 16>(a, st);

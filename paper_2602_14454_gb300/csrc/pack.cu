@@ -201,15 +201,49 @@ struct Dims {
 };
 constexpr int kLinks = 128;   // links per CTA: 16 sites of one parity, 8 directions
 
+// A link for the fixed-point hop: entries U 2^(e - 59) as limbs {re low, re high, im
+// low, im high} (fx_limbs31s), nine per link, and its exponent or mark.
+__device__ __forceinline__ int link_exponent(const double2 *u)
+{
+    uint32_t m = 0, low = 0;
+#pragma unroll
+    for (int k = 0; k < 9; ++k) {
+        m = max(m, max((uint32_t)__double2hiint(u[k].x) & 0x7fffffffu, (uint32_t)__double2hiint(u[k].y) & 0x7fffffffu));
+        low |= (uint32_t)__double2loint(u[k].x) | (uint32_t)__double2loint(u[k].y);
+    }
+    return fx_exponent(m, low);
+}
+__device__ __forceinline__ int4 link_limbs(double2 q, int e)
+{
+    int4 w;
+    fx_limbs31s(fx_from_double(q.x, e, FX_BITS), w.x, w.y);
+    fx_limbs31s(fx_from_double(q.y, e, FX_BITS), w.z, w.w);
+    return w;
+}
+// the same from an FP64 copy (a slab's)
+__global__ void __launch_bounds__(128) links_to_limbs_kernel(const double2 *g64, int4 *gfx, int *ge, size_t n)
+{
+    for (size_t l = blockIdx.x * (size_t)blockDim.x + threadIdx.x; l < n; l += (size_t)gridDim.x * blockDim.x) {
+        double2 u[9];
+#pragma unroll
+        for (int k = 0; k < 9; ++k) u[k] = g64[l * 9 + k];
+        const int e = link_exponent(u);
+        ge[l] = e;
+#pragma unroll
+        for (int k = 0; k < 9; ++k) gfx[l * 9 + k] = link_limbs(u[k], e);
+    }
+}
+
 // Neighbouring CTAs take the two parities of the same sites, so that most of a
 // link's second read (it belongs to both of its ends) comes from L2.
 __global__ void __launch_bounds__(kLinks) pack_gauge_kernel(const double *U, Dims D, int Vh, double2 *g64, float4 *g32,
-                                                            uint4 *g16)
+                                                            uint4 *g16, int4 *gfx, int *ge)
 {
     __shared__ __align__(16) double2 u[kLinks * 9];
     __shared__ const double2 *from[kLinks];
     __shared__ bool minus[kLinks];   // the boundary phase is -1
     __shared__ bool dagger[kLinks];
+    __shared__ int eu[kLinks];
     const int par = blockIdx.x & 1, tid = threadIdx.x;
     const long long first = (long long)(blockIdx.x >> 1) * kLinks, total = (long long)Vh * 8;
     const int n = (int)min((long long)kLinks, total - first);
@@ -248,6 +282,16 @@ __global__ void __launch_bounds__(kLinks) pack_gauge_kernel(const double *U, Dim
     }
     __syncthreads();
     const size_t out = (size_t)par * total + first;   // this CTA's first link
+    if (tid < n) {
+        eu[tid] = link_exponent(u + tid * 9);
+        ge[out + tid] = eu[tid];
+    }
+    __syncthreads();
+#pragma unroll
+    for (int j = 0; j < 9; ++j) {
+        const int f = tid + j * kLinks;
+        if (f < n * 9) gfx[out * 9 + f] = link_limbs(u[f], eu[f / 9]);
+    }
 #pragma unroll
     for (int j = 0; j < 9; ++j) {
         const int f = tid + j * kLinks;
@@ -365,14 +409,21 @@ cudaError_t launch_pack_mix(int prec, const double *canon, FieldRef x, const Mix
     return cudaErrorInvalidValue;
 }
 
+cudaError_t launch_links_to_limbs(const void *g64, int4 *gfx, int *ge, size_t n, cudaStream_t st)
+{
+    const size_t b = (n + 127) / 128;
+    links_to_limbs_kernel<<<(unsigned)(b < 152 * 64 ? b : 152 * 64), 128, 0, st>>>((const double2 *)g64, gfx, ge, n);
+    return cudaGetLastError();
+}
+
 cudaError_t launch_pack_gauge(const double *U, const int dims[4], const int bc[4], void *g64, void *g32, void *g16,
-                              cudaStream_t st)
+                              int4 *gfx, int *ge, cudaStream_t st)
 {
     Dims D;
     for (int k = 0; k < 4; ++k) D.d[k] = dims[k], D.bc[k] = bc[k];
     const int Vh = dims[0] * dims[1] * dims[2] * dims[3] / 2;
     const unsigned g = (unsigned)(2 * (((long long)Vh * 8 + kLinks - 1) / kLinks));
-    pack_gauge_kernel<<<g, kLinks, 0, st>>>(U, D, Vh, (double2 *)g64, (float4 *)g32, (uint4 *)g16);
+    pack_gauge_kernel<<<g, kLinks, 0, st>>>(U, D, Vh, (double2 *)g64, (float4 *)g32, (uint4 *)g16, gfx, ge);
     return cudaGetLastError();
 }
 
