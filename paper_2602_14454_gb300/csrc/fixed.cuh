@@ -69,17 +69,22 @@ FX_HD int fx_clz(uint64_t x)
 #endif
 }
 
-// R 2^s as a double, rounded once to nearest even (twice below FP64's normal range).
-// In integers: the conversion instruction runs on the FP64 pipe.
-FX_HD double fx_to_double(int64_t R, int s)
+// R 2^s as a double for -1000 < s < 950, where it is normal, rounded once to nearest
+// even.  In integers: the conversion instruction runs on the FP64 pipe.
+FX_HD constexpr bool fx_normal_shift(int s) { return s > -1000 && s < 950; }
+FX_HD double fx_to_double_normal(int64_t R, int s)
 {
     const uint64_t sg = (uint64_t)(R >> 63), a = ((uint64_t)R ^ sg) - sg;
     const int z = fx_clz(a);
-    if (s <= -1000 || s >= 950) return scalbn((double)R, s);
     const uint64_t v = a << ((z - 1) & 63);   // leading bit at 62
     const uint64_t r = (v + 0x1ff + ((v >> 10) & 1)) >> 10;
     const uint64_t e = (uint64_t)(uint32_t)(1085 + s - z) << 52;   // r's bit 52 adds the last one
     return fx_of_bits(a ? (int64_t)((e + r) | (sg << 63)) : 0);
+}
+// any s (rounded twice below FP64's normal range)
+FX_HD double fx_to_double(int64_t R, int s)
+{
+    return fx_normal_shift(s) ? fx_to_double_normal(R, s) : scalbn((double)R, s);
 }
 
 // The exponent field of the largest of the doubles whose high words' magnitudes

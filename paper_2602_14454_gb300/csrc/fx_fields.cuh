@@ -62,12 +62,28 @@ __device__ __forceinline__ int fx_pack(const double2 *v, int B, longlong2 *t)
                            : make_longlong2(fx_from_double(v[k].x, e, B), fx_from_double(v[k].y, e, B));
     return e;
 }
-__device__ __forceinline__ void fx_unpack(const longlong2 *t, int e, int B, double2 *v)
+// one value of a marked block, or of one whose exponent leaves FP64's normal range: out
+// of line, as 24 inlined scalings would crowd the instruction cache
+__device__ __noinline__ double fx_value_rare(long long r, int s, bool raw)
 {
+    return raw ? __longlong_as_double(r) : fx_to_double(r, s);
+}
+// v = r 2^(s0 or s1 by chirality), or the raw doubles
+__device__ __forceinline__ void fx_to_doubles(const longlong2 *r, int s0, int s1, bool raw, double2 *v)
+{
+    if (!raw && fx_normal_shift(s0) && fx_normal_shift(s1)) {
 #pragma unroll
-    for (int k = 0; k < 12; ++k)
-        v[k] = e == FX_RAW ? make_double2(__longlong_as_double(t[k].x), __longlong_as_double(t[k].y))
-                           : make_double2(fx_to_double(t[k].x, e - B), fx_to_double(t[k].y, e - B));
+        for (int k = 0; k < 12; ++k) {
+            const int s = k & 1 ? s1 : s0;
+            v[k] = make_double2(fx_to_double_normal(r[k].x, s), fx_to_double_normal(r[k].y, s));
+        }
+    } else {
+#pragma unroll
+        for (int k = 0; k < 12; ++k) {
+            const int s = k & 1 ? s1 : s0;
+            v[k] = make_double2(fx_value_rare(r[k].x, s, raw), fx_value_rare(r[k].y, s, raw));
+        }
+    }
 }
 // v[12] <- an FP64 or block field as doubles
 template <bool RO>
@@ -76,7 +92,8 @@ __device__ __forceinline__ void fx_ld_double(const FieldRef &f, size_t site, int
     if (f.fx) {
         longlong2 t[12];
         fx_ld<RO>(f, site, s, Ls, t);
-        fx_unpack(t, f.fx[site * Ls + s], FX_BITS, v);
+        const int e = f.fx[site * Ls + s];
+        fx_to_doubles(t, e - FX_BITS, e - FX_BITS, e == FX_RAW, v);
     } else {
         ld_pairs<DWF_F64, RO>(f, site, s, Ls, v);
     }
@@ -244,11 +261,9 @@ __device__ __forceinline__ void fx_mix(const FxMat &M, const int4 *tile, const i
     fx_mix_chi<0>(M, tile, te, s, Ls, S.E[0], S.r);
     fx_mix_chi<1>(M, tile, te, s, Ls, S.E[1], S.r);
 }
-__device__ __forceinline__ double2 fx_sum_double(const FxSum &S, int k, int B)
+__device__ __forceinline__ void fx_sum_doubles(const FxSum &S, int B, double2 *o)
 {
-    if (S.raw) return make_double2(__longlong_as_double(S.r[k].x), __longlong_as_double(S.r[k].y));
-    const int e = S.E[k & 1] + 58 - 2 * B;
-    return make_double2(fx_to_double(S.r[k].x, e), fx_to_double(S.r[k].y, e));
+    fx_to_doubles(S.r, S.E[0] + 58 - 2 * B, S.E[1] + 58 - 2 * B, S.raw, o);
 }
 // S += T; both below 2^62 in magnitude, and so is the sum
 __device__ __forceinline__ void fx_sum_add(FxSum &S, const FxSum &T, int B)
@@ -256,7 +271,9 @@ __device__ __forceinline__ void fx_sum_add(FxSum &S, const FxSum &T, int B)
     if (S.raw || T.raw) {
 #pragma unroll
         for (int k = 0; k < 12; ++k) {
-            const double2 q = p_add(fx_sum_double(S, k, B), fx_sum_double(T, k, B));
+            const int a = S.E[k & 1] + 58 - 2 * B, b = T.E[k & 1] + 58 - 2 * B;
+            const double2 q = make_double2(fx_value_rare(S.r[k].x, a, S.raw) + fx_value_rare(T.r[k].x, b, T.raw),
+                                           fx_value_rare(S.r[k].y, a, S.raw) + fx_value_rare(T.r[k].y, b, T.raw));
             S.r[k] = make_longlong2(__double_as_longlong(q.x), __double_as_longlong(q.y));
         }
         S.raw = true;
@@ -288,8 +305,7 @@ __device__ __forceinline__ void fx_store_sum(const FieldRef &out, size_t site, i
 {
     if (!out.fx || S.raw) {
         double2 o[12];
-#pragma unroll
-        for (int k = 0; k < 12; ++k) o[k] = fx_sum_double(S, k, B);
+        fx_sum_doubles(S, B, o);
         fx_store_double(out, site, s, Ls, o);
         return;
     }

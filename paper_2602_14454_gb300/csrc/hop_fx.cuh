@@ -283,8 +283,7 @@ __global__ void __launch_bounds__(128, 4) hop_fx_kernel(const HopArgs a)
     double2 o[12];
     double nrm = 0;
     if (active) {
-#pragma unroll
-        for (int k = 0; k < 12; ++k) o[k] = fx_sum_double(S, k, B);
+        fx_sum_doubles(S, B, o);
         if (a.ymode == 1) {
             double2 y[12];
             fx_ld_double<false>(a.y, (size_t)site, s, Ls, y);
