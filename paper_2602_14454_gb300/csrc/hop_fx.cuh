@@ -14,8 +14,9 @@
 //
 // Bound: the multiply pipe, 216 multiply-adds of four cycles per direction and warp,
 // closely followed by the integer adds and shifts (342 of two cycles) and the issue
-// slots; DRAM is 15 % busy.  At 16^3x32, Ls 16 (K_a, dense mixing): 502 us against
-// 1987 us on the FP64 pipe, of which the eight directions 267 us, the mixing 155 us.
+// slots; DRAM is 15 % busy.  At 16^3x32, Ls 16 (K_a, dense mixing): 485 us against
+// 1987 us on the FP64 pipe, of which the eight directions 267 us, the mixing about
+// 150 us (there the shared-memory reads bound it: 39 wavefronts per (site, s)).
 #pragma once
 
 #include "fx_fields.cuh"   // before stencil.cuh: its templates take the integer pairs
