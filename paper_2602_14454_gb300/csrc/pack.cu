@@ -317,9 +317,9 @@ __global__ void __launch_bounds__(kLinks) pack_gauge_kernel(const double *U, Dim
 // P_+ b4 and P_- b4.  Thread per (lexicographic site, slice).
 __global__ void __launch_bounds__(128) walls_kernel(const double *b4, FieldRef even, FieldRef odd, const int *eo2lex, int V)
 {
-    const int f = blockIdx.x * blockDim.x + threadIdx.x;
-    if (f >= 2 * V) return;
-    const int lex = f >> 1, w = f & 1, i = lex >> 1;
+    const size_t f = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
+    if (f >= (size_t)2 * V) return;
+    const int lex = (int)(f >> 1), w = (int)(f & 1), i = lex >> 1;
     const double *c = b4 + (size_t)lex * 24;
     double2 v[12];
 #pragma unroll
@@ -339,8 +339,9 @@ __global__ void source_canon_kernel(const double *b4, FieldRef he, FieldRef ho, 
 {
     const size_t f = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
     if (f >= (size_t)V * 24) return;
-    const int w = f >= (size_t)V * 12, r = (int)(f - (w ? (size_t)V * 12 : 0));
-    const int lex = r / 12, k = r - lex * 12, spin = k / 3, a = k - spin * 3, i = lex >> 1;
+    const int w = f >= (size_t)V * 12;
+    const size_t r = f - (w ? (size_t)V * 12 : 0);
+    const int lex = (int)(r / 12), k = (int)(r - (size_t)lex * 12), spin = k / 3, a = k - spin * 3, i = lex >> 1;
     const double *h = reinterpret_cast<const double *>((lex == __ldg(eo2lex + i) ? he : ho).v);
     // the reals (re, im) of (spin, a): groups 2 a and 2 a + 1, pair spin >> 1 of the group
     const size_t at = (((size_t)i * 12 + 4 * a + (spin >> 1)) * 2 + w) * 2 + (spin & 1);
