@@ -455,12 +455,15 @@ static int solve_impl(dwf_handle h, const void *b5, void *x5, const dwf_solve_pa
     // graph of N inner iterations
     GraphCache &G = X.graph;
     char keybuf[256];
-    // the captured kernels depend on the hop configuration and mixing mode too
-    std::snprintf(keybuf, sizeof keybuf, "%d/%d/%p/%p/%p/%d/%d/%d/%d/%d/%d/%d", ps, N, B.p.v, B.rs.v, B.xs.v,
-                  p->use_graph, h->hop_var[ps], h->hop_ns[ps], h->hop_sb[ps], h->mix_mode(ps), B.form, (int)B.fx);
+    // the captured kernels depend on the hop configuration, the mixing mode (as set: the default
+    // chooses by operation) and the sweep order too
+    std::snprintf(keybuf, sizeof keybuf, "%d/%d/%p/%p/%p/%d/%d/%d/%d/%d/%d/%d/%d", ps, N, B.p.v, B.rs.v, B.xs.v,
+                  p->use_graph, h->hop_var[ps], h->hop_ns[ps], h->hop_sb[ps], h->mixmode[ps], h->sweep_zb[ps], B.form,
+                  (int)B.fx);
     if (p->use_graph && G.key != keybuf) {
         if (G.exec) cudaGraphExecDestroy(G.exec);
         G.exec = nullptr;
+        G.key.clear();   // no graph until the capture below succeeds
         cudaGraph_t g;
         const long long saved = h->launches;
         CK(cudaStreamBeginCapture(X.cap, cudaStreamCaptureModeThreadLocal));
