@@ -378,7 +378,10 @@ long long dwf_launch_count(dwf_handle h);
  * which dwf_get_hop_config answers 0; any variant or mixing mode chosen for
  * FP64 selects the FP64 arithmetic instead).  Variants differ only in the order
  * of the sums, except 5 (FP16 rounding of the projection), 10 (products of the
- * TF32 terms) and the FP64 default (its own rounding, below FP64's).  Numbers 1, 2, 6 and 8 are not used.
+ * TF32 terms) and the FP64 default, whose errors are relative to the largest
+ * entry of each (site, s, chirality) and of each link: in the norm of those not
+ * above FP64's, but an entry 2^-k below the largest keeps 59 - k bits (55 - k
+ * at least), where FP64 keeps 53.  Numbers 1, 2, 6 and 8 are not used.
  * Errors: DWF_EINVAL (NULL handle or pointer, bad prec, variant not -1, 0, 3,
  * 4, 5, 7, 9 or 10, ns or sb outside the ranges above, sb making a CTA of more
  * than 256 threads). */

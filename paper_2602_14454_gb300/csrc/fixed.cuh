@@ -3,17 +3,25 @@
 // GB300 issues two FP64 operations per clock and SM (measured: 1.98 DFMA lanes) but
 // about 32 integer multiply-adds 32 x 32 + 64 -> 64 (the counters show four cycles
 // of the multiply pipe per warp), so the products of the FP64 hop and of its
-// fifth-direction mixing run on the integer pipe.  A block is the 24 reals x_k of one (site, s):
+// fifth-direction mixing run on the integer pipe.  A block is the 24 reals of one
+// (site, s), in two halves by chirality, P_+ and P_- (12 reals each: the fifth
+// direction's matrices mix slices of one chirality and never the two):
 //     x_k = F_k 2^(e - 59),  F_k integers below 2^59 in magnitude,
-// e the block's exponent (every |x_k| < 2^e, the largest at least 2^(e - 1)).
+// e the half's exponent (every |x_k| < 2^e, the largest at least 2^(e - 1); in fields
+// at least 2^(e - 5), see fx_near).
 // A product takes two limbs per factor and three multiply-adds (hi hi and the two
 // cross products; lo lo lies below the kept bits), sums are exact integer
-// additions, and one rounding to FP64 follows at the end.  Where FP64 keeps 53
-// bits of every number, a block keeps 59 bits relative to its largest: its
-// rounding errors are the smaller ones in the norm of every (site, s).
+// additions, and one rounding to FP64 follows at the end.
 //
-// A block with an infinite or NaN entry is marked by e = FX_RAW and holds the
-// doubles' own bits; a kernel that reads a marked block computes the sites it
+// Accuracy: FP64 keeps 53 bits of every number, a half block 55 to 59 bits relative to
+// its largest.  Its errors are the smaller ones wherever the terms of an output are of
+// the half blocks' size, so in the norm of every half block for links that mix
+// colours; an entry 2^-k below the largest of its own half block keeps k bits less.
+// Products that must keep entries of one half block apart by more than that (unit
+// links, colours of very different size) take the FP64 kernels (hop variant 0).
+//
+// A block with an infinite or NaN entry is marked by e = FX_RAW in both halves and
+// holds the doubles' own bits; a kernel that reads a marked block computes the sites it
 // reaches in FP64, so non-finite values spread as FP64 arithmetic spreads them.
 //
 // Everything here is 64-bit integer C++ that also runs on the host.
@@ -34,6 +42,16 @@ namespace dwf {
 constexpr int FX_BITS = 59;
 constexpr int FX_RAW = 0x4000;     // the block holds raw doubles
 constexpr int FX_ZERO = -0x4000;   // every entry is zero
+
+// The exponents of a block's halves in one word, P_+ in the low 16 bits.  Doubles,
+// links and constants have exponents within 1100; two hops with their mixings (no
+// field is held in blocks for longer) stay within 6000, so no exponent comes near the
+// marks, and marked words compare above all others.
+FX_HD constexpr int fx_word(int ep, int em) { return (int)((uint32_t)em << 16 | ((uint32_t)ep & 0xffffu)); }
+template <int CHI>
+FX_HD constexpr int fx_half(int word) { return CHI ? word >> 16 : (int)(int16_t)(uint16_t)(uint32_t)word; }
+constexpr int FX_RAW_BLOCK = fx_word(FX_RAW, FX_RAW);
+FX_HD constexpr bool fx_is_raw(int word) { return word >= FX_RAW_BLOCK - FX_RAW; }
 
 // Bits of a mixing tile's entries and of the mixing constants: the sums over Ls
 // slices of hi hi and of the cross products (radix 2^29) stay below 2^63.
@@ -58,6 +76,16 @@ FX_HD double fx_of_bits(int64_t b)
     std::memcpy(&x, &b, 8);
     return x;
 #endif
+}
+// Halves of a field whose exponents differ by at most 4 take the larger one: the other
+// half keeps 55 bits or more, and a hop, which adds the two halves, need not shift them
+// against one another (even-odd application at 16^3x32, Ls 16: 1229 us, and 1275 us
+// where every block's halves lie 20 bits apart).
+constexpr int FX_NEAR = 4;
+FX_HD void fx_near(int &ep, int &em)
+{
+    const int top = ep > em ? ep : em;
+    if (top - ep <= FX_NEAR && top - em <= FX_NEAR) ep = em = top;
 }
 // number of leading zeros; 64 for 0
 FX_HD int fx_clz(uint64_t x)

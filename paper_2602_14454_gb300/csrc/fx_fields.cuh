@@ -3,10 +3,10 @@
 // fixed.cuh, field layout in dwf_internal.h).
 //
 // A block field stores the field's 16-byte vectors with 64-bit integers in the
-// place of the doubles, and one exponent per (site, s), [site][Ls] int32, behind
-// it (FieldRef::fx).  Registers hold a block as 12 pairs in the order of the FP64
-// kernels (even pairs P_+, odd pairs P_-), so project() and reconstruct() of
-// stencil.cuh apply to it as they are.
+// place of the doubles, and one word of two exponents (fx_word) per (site, s),
+// [site][Ls], behind it (FieldRef::fx).  Registers hold a block as 12 pairs in the
+// order of the FP64 kernels (even pairs P_+, odd pairs P_-), so project() and
+// reconstruct() of stencil.cuh apply to it once both halves have one exponent.
 #pragma once
 
 #include "fields.cuh"
@@ -41,26 +41,32 @@ __device__ __forceinline__ void fx_st(const FieldRef &f, size_t site, int s, int
     f.fx[site * Ls + s] = e;
 }
 
-// the exponent (or mark) of 12 pairs of doubles
-__device__ __forceinline__ int fx_block_exponent(const double2 *v)
+// the exponent (or mark) of the pairs of chirality CHI
+template <int CHI>
+__device__ __forceinline__ int fx_half_exponent(const double2 *v)
 {
     uint32_t m = 0, low = 0;
 #pragma unroll
-    for (int k = 0; k < 12; ++k) {
+    for (int k = CHI; k < 12; k += 2) {
         m = max(m, max((uint32_t)__double2hiint(v[k].x) & 0x7fffffffu, (uint32_t)__double2hiint(v[k].y) & 0x7fffffffu));
         low |= (uint32_t)__double2loint(v[k].x) | (uint32_t)__double2loint(v[k].y);
     }
     return fx_exponent(m, low);
 }
-// doubles -> integers of B bits below 2^e; a marked block keeps the doubles' bits
+// doubles -> integers of B bits below 2^e, e of each half (B = FX_BITS: of a field);
+// a marked block keeps the doubles' bits.  Returns the exponents' word.
 __device__ __forceinline__ int fx_pack(const double2 *v, int B, longlong2 *t)
 {
-    const int e = fx_block_exponent(v);
+    int ep = fx_half_exponent<0>(v), em = fx_half_exponent<1>(v);
+    const bool raw = max(ep, em) == FX_RAW;
+    if (B == FX_BITS) fx_near(ep, em);
 #pragma unroll
-    for (int k = 0; k < 12; ++k)
-        t[k] = e == FX_RAW ? make_longlong2(__double_as_longlong(v[k].x), __double_as_longlong(v[k].y))
-                           : make_longlong2(fx_from_double(v[k].x, e, B), fx_from_double(v[k].y, e, B));
-    return e;
+    for (int k = 0; k < 12; ++k) {
+        const int e = k & 1 ? em : ep;
+        t[k] = raw ? make_longlong2(__double_as_longlong(v[k].x), __double_as_longlong(v[k].y))
+                   : make_longlong2(fx_from_double(v[k].x, e, B), fx_from_double(v[k].y, e, B));
+    }
+    return raw ? FX_RAW_BLOCK : fx_word(ep, em);
 }
 // one value of a marked block, or of one whose exponent leaves FP64's normal range: out
 // of line, as 24 inlined scalings would crowd the instruction cache
@@ -93,20 +99,20 @@ __device__ __forceinline__ void fx_ld_double(const FieldRef &f, size_t site, int
         longlong2 t[12];
         fx_ld<RO>(f, site, s, Ls, t);
         const int e = f.fx[site * Ls + s];
-        fx_to_doubles(t, e - FX_BITS, e - FX_BITS, e == FX_RAW, v);
+        fx_to_doubles(t, fx_half<0>(e) - FX_BITS, fx_half<1>(e) - FX_BITS, fx_is_raw(e), v);
     } else {
         ld_pairs<DWF_F64, RO>(f, site, s, Ls, v);
     }
 }
 
-// bits of the largest of the pairs k = first, first + step, ...
-template <int STEP>
-__device__ __forceinline__ int fx_pairs_width(const longlong2 *v, int first)
+// bits of the largest of the pairs of chirality CHI
+template <int CHI>
+__device__ __forceinline__ int fx_half_width(const longlong2 *v)
 {
     uint32_t hi = 0, lo = 0;
 #pragma unroll
-    for (int k = 0; k < 12; k += STEP) {
-        const longlong2 q = v[k + first];
+    for (int k = CHI; k < 12; k += 2) {
+        const longlong2 q = v[k];
         const int32_t hx = (int32_t)(q.x >> 32), hy = (int32_t)(q.y >> 32);
         hi |= (uint32_t)(hx ^ (hx >> 31)) | (uint32_t)(hy ^ (hy >> 31));
         lo |= (uint32_t)((int32_t)q.x ^ (hx >> 31)) | (uint32_t)((int32_t)q.y ^ (hy >> 31));
@@ -115,19 +121,21 @@ __device__ __forceinline__ int fx_pairs_width(const longlong2 *v, int first)
     const int w = hi ? 64 - __clz((int)hi) : 32 - __clz((int)lo);
     return w > 0 ? w : 1;
 }
-__device__ __forceinline__ bool fx_all_zero(const longlong2 *v)
+// all pairs of chirality CHI zero
+template <int CHI>
+__device__ __forceinline__ bool fx_half_zero(const longlong2 *v)
 {
     unsigned long long any = 0;
 #pragma unroll
-    for (int k = 0; k < 12; ++k) any |= (unsigned long long)v[k].x | (unsigned long long)v[k].y;
+    for (int k = CHI; k < 12; k += 2) any |= (unsigned long long)v[k].x | (unsigned long long)v[k].y;
     return any == 0;
 }
 
 // ------------------------------------------------------------------ the tile
 // Tile rows of one (site, s): 12 vectors of 16 bytes, each two reals as limbs
 // (low, high; radix 2^29), rows 13 vectors apart so that eight lanes' 16-byte
-// accesses hit distinct banks; te[site row] the exponents.  A marked row holds
-// raw doubles.
+// accesses hit distinct banks; te[site row] the exponents' words.  A marked row
+// holds raw doubles.
 constexpr int FX_ROW = 13;
 __host__ __device__ constexpr int fx_site_stride(int Ls) { return Ls * FX_ROW + 1; }
 
@@ -136,7 +144,7 @@ __device__ __forceinline__ void fx_put(int4 *row, const longlong2 *t, int e)
 #pragma unroll
     for (int k = 0; k < 12; ++k) {
         int4 q;
-        if (e == FX_RAW) {
+        if (fx_is_raw(e)) {
             q = make_int4((int)t[k].x, (int)(t[k].x >> 32), (int)t[k].y, (int)(t[k].y >> 32));
         } else {
             fx_limbs29(t[k].x, q.x, q.y);
@@ -145,9 +153,10 @@ __device__ __forceinline__ void fx_put(int4 *row, const longlong2 *t, int e)
         row[k] = q;
     }
 }
-__device__ __forceinline__ double fx_tile_double(int lo, int hi, int e, int B)
+__device__ __forceinline__ double fx_tile_double(int lo, int hi, int e, int chi, int B)
 {
-    return e == FX_RAW ? __hiloint2double(hi, lo) : fx_to_double(((int64_t)hi << 29) + lo, e - B);
+    return fx_is_raw(e) ? __hiloint2double(hi, lo)
+                        : fx_to_double(((int64_t)hi << 29) + lo, (chi ? fx_half<1>(e) : fx_half<0>(e)) - B);
 }
 
 // A fifth-direction matrix: constants {mantissa low, high word, exponent, 0} of B
@@ -158,28 +167,28 @@ struct FxMat {
     int band;   // 0 dense, 1 cyclic tridiagonal, 2 diagonal
 };
 
-// E[chi] of output s: the largest exponent of M_st x_t over the rows t; also the
-// largest row exponent, for the mark.
-__device__ __forceinline__ int fx_mix_exponents(const FxMat &M, const int *te, int s, int Ls, int *E)
+// E[chi] of output s: the largest exponent of M_st x_t over the rows t; returns
+// whether a row is marked.
+__device__ __forceinline__ bool fx_mix_exponents(const FxMat &M, const int *te, int s, int Ls, int *E)
 {
     const int n = M.band == 0 ? Ls : (M.band == 1 ? 3 : 1);
-    int t = M.band == 1 ? (s ? s - 1 : Ls - 1) : s, mark = FX_ZERO;
+    int t = M.band == 1 ? (s ? s - 1 : Ls - 1) : s, mark = 0;
     const int4 *c = M.c + s;
     E[0] = E[1] = 2 * FX_ZERO;
 #pragma unroll 4
     for (int i = 0; i < n; ++i) {
         const int e = te[t];
         mark = max(mark, e);
-        E[0] = max(E[0], __ldg(&c[t * Ls].z) + e);
-        E[1] = max(E[1], __ldg(&c[(Ls + t) * Ls].z) + e);
+        E[0] = max(E[0], __ldg(&c[t * Ls].z) + fx_half<0>(e));
+        E[1] = max(E[1], __ldg(&c[(Ls + t) * Ls].z) + fx_half<1>(e));
         t = t + 1 < Ls ? t + 1 : 0;
     }
-    return mark;
+    return fx_is_raw(mark);
 }
 
 // r[k] (pairs of chirality CHI only): (M tile)(s) = r 2^(E + 58 - 2 B).  Every product
-// M_st x_t is taken against E by shifting the constant, so a small row next to large
-// ones loses nothing that FP64 would have kept.  Constants that vanish there are
+// M_st x_t is taken against E by shifting the constant: a row of small half blocks
+// keeps its bits where it meets the large ones of other rows.  Constants that vanish there are
 // skipped, and those below 2^28 take one multiply-add instead of three: the
 // inverse's entries fall off by a factor kappa per slice (0.023 for b 1.5, c 0.5).
 // Lane s starts at row s, so that a warp meets constants of one size together.
@@ -190,6 +199,7 @@ __device__ __forceinline__ void fx_mix_chi(const FxMat &M, const int4 *tile, con
     const int n = M.band == 0 ? Ls : (M.band == 1 ? 3 : 1);
     int t = M.band == 1 ? (s ? s - 1 : Ls - 1) : s;
     const int4 *c = M.c + CHI * Ls * Ls + s;
+    const short *te2 = reinterpret_cast<const short *>(te) + CHI;   // one half of each word
     int64_t hh[12], x[12];
 #pragma unroll
     for (int k = 0; k < 12; ++k) hh[k] = 0, x[k] = 1 << 28;   // the cross sums are rounded at 2^29
@@ -197,7 +207,7 @@ __device__ __forceinline__ void fx_mix_chi(const FxMat &M, const int4 *tile, con
 #pragma unroll 1
     for (int i = 0; i < n; ++i) {
         const int4 q = next;
-        const int sh = E - (q.z + te[t]);
+        const int sh = E - (q.z + te2[2 * t]);
         const int4 *row = tile + t * FX_ROW + CHI;
         t = t + 1 < Ls ? t + 1 : 0;
         next = __ldg(&c[t * Ls]);
@@ -237,8 +247,8 @@ __device__ __noinline__ void fx_mix_raw(const FxMat &M, const int4 *tile, const 
             const double m = M.m[(size_t)(k & 1) * Ls * Ls + (size_t)t * Ls + s];
             if (m == 0.0) continue;   // a row that the matrix does not couple
             const int4 q = tile[t * FX_ROW + k];
-            o[k].x = fma(m, fx_tile_double(q.x, q.y, te[t], B), o[k].x);
-            o[k].y = fma(m, fx_tile_double(q.z, q.w, te[t], B), o[k].y);
+            o[k].x = fma(m, fx_tile_double(q.x, q.y, te[t], k & 1, B), o[k].x);
+            o[k].y = fma(m, fx_tile_double(q.z, q.w, te[t], k & 1, B), o[k].y);
         }
     }
 }
@@ -252,7 +262,7 @@ struct FxSum {
 };
 __device__ __forceinline__ void fx_mix(const FxMat &M, const int4 *tile, const int *te, int s, int Ls, int B, FxSum &S)
 {
-    S.raw = fx_mix_exponents(M, te, s, Ls, S.E) >= FX_RAW;
+    S.raw = fx_mix_exponents(M, te, s, Ls, S.E);
     if (S.raw) {
         double2 o[12];
         fx_mix_raw(M, tile, te, s, Ls, B, o);
@@ -311,15 +321,18 @@ __device__ __forceinline__ void fx_store_sum(const FieldRef &out, size_t site, i
         fx_store_double(out, site, s, Ls, o);
         return;
     }
-    const int w[2] = {fx_pairs_width<2>(S.r, 0), fx_pairs_width<2>(S.r, 1)};
-    const int top[2] = {w[0] + S.E[0] + 58 - 2 * B, w[1] + S.E[1] + 58 - 2 * B};   // |value| < 2^top
-    const int e = max(top[0], top[1]);
+    const int wp = fx_half_width<0>(S.r), wm = fx_half_width<1>(S.r);
+    // |value| < 2^top
+    const int tp = fx_half_zero<0>(S.r) ? FX_ZERO : wp + S.E[0] + 58 - 2 * B;
+    const int tm = fx_half_zero<1>(S.r) ? FX_ZERO : wm + S.E[1] + 58 - 2 * B;
+    int ep = tp, em = tm;
+    fx_near(ep, em);
 #pragma unroll
     for (int k = 0; k < 12; ++k) {
-        const int c = k & 1, down = 63 - FX_BITS + (e - top[c]);
-        S.r[k] = make_longlong2(fx_align(S.r[k].x, w[c], down), fx_align(S.r[k].y, w[c], down));
+        const int w = k & 1 ? wm : wp, down = 63 - FX_BITS + (k & 1 ? em - tm : ep - tp);
+        S.r[k] = make_longlong2(fx_align(S.r[k].x, w, down), fx_align(S.r[k].y, w, down));
     }
-    fx_st(out, site, s, Ls, S.r, fx_all_zero(S.r) ? FX_ZERO : e);
+    fx_st(out, site, s, Ls, S.r, fx_word(ep, em));
 }
 
 }  // namespace

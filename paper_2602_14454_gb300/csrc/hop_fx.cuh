@@ -9,14 +9,16 @@
 // no longer fits the instruction cache): each has its neighbour's block copied
 // asynchronously into its own shared slots one direction ahead, projects, multiplies
 // and reconstructs in integers.  The eight directions' exponents are known before
-// the first product (block exponent + link exponent), so all are summed against the
+// the first product (the larger half's + link exponent), so all are summed against the
 // largest.
 //
 // Bound: the multiply pipe, 216 multiply-adds of four cycles per direction and warp,
 // closely followed by the integer adds and shifts (342 of two cycles) and the issue
-// slots; DRAM is 15 % busy.  At 16^3x32, Ls 16 (K_a, dense mixing): 485 us against
-// 1987 us on the FP64 pipe, of which the eight directions 267 us, the mixing about
-// 150 us (there the shared-memory reads bound it: 39 wavefronts per (site, s)).
+// slots; DRAM is 15 % busy.  At 16^3x32, Ls 16 (K_a, dense mixing): 498 us against
+// 1987 us on the FP64 pipe (485 us with one exponent for both halves of a block).  In
+// an earlier form of 502 us (links made into limbs here) the eight directions took
+// about 267 us and the mixing about 155 us, bound by its shared-memory reads.  All
+// forms use 128 registers and spill 250 to 432 bytes a thread.
 #pragma once
 
 #include "fx_fields.cuh"   // before stencil.cuh: its templates take the integer pairs
@@ -105,6 +107,17 @@ __device__ __forceinline__ void fx_fetch(int4 *slot, int nt, const FieldRef &in,
     for (int k = 0; k < 12; ++k)
         asm volatile("cp.async.ca.shared.global [%0], [%1], 16;" ::"r"(d + k * nt * 16), "l"(p + (size_t)k * Ls) : "memory");
     asm volatile("cp.async.commit_group;" ::: "memory");
+}
+
+// the half of a block in its slots that lies lower, by |above| bits, shifted to the
+// other's exponent; out of line, as fields seldom need it (fx_near)
+__device__ __noinline__ void fx_even_halves(int4 *slot, int nt, int above)
+{
+    const int c = above > 0, sh = above > 0 ? above : -above;
+    for (int k = c; k < 12; k += 2) {
+        longlong2 *q = reinterpret_cast<longlong2 *>(slot + k * nt);
+        *q = make_longlong2(q->x >> sh, q->y >> sh);
+    }
 }
 
 // one direction in FP64, for sites with non-finite neighbours or links
@@ -198,25 +211,37 @@ __global__ void __launch_bounds__(128, 4) hop_fx_kernel(const HopArgs a)
     __syncthreads();
 
     longlong2 acc[12];
-    int emax = 2 * FX_ZERO, mark = FX_ZERO;
+    int emax = 2 * FX_ZERO;
+    bool raw = false;
 #pragma unroll
     for (int k = 0; k < 12; ++k) acc[k] = make_longlong2(0, 0);
     if (active) {
+        uint64_t shifts = 0, above = 0;   // eight bits per direction: emax - e, at most 63, and how far P_+ lies above P_-
+        bool uneven = false;
 #pragma unroll
         for (int d = 0; d < 8; ++d) {
-            const int eu = sm.eu[j * 8 + d];
-            mark = max(mark, max(e8[d], eu));
-            e8[d] += eu;
+            const int eu = sm.eu[j * 8 + d], ep = fx_half<0>(e8[d]), em = fx_half<1>(e8[d]);
+            raw = raw || fx_is_raw(e8[d]) || eu == FX_RAW;
+            uneven = uneven || ep != em;
+            e8[d] = max(ep, em) + eu;
             emax = max(emax, e8[d]);
         }
-        uint64_t shifts = 0;   // emax - e per direction, at most 63, eight bits each
 #pragma unroll
         for (int d = 0; d < 8; ++d) shifts |= (uint64_t)(uint32_t)min(emax - e8[d], 63) << (8 * d);
+        if (uneven) {   // rare in fields (fx_near): projecting takes both halves at the larger exponent
+#pragma unroll 1
+            for (int d = 0; d < 8; ++d) {
+                const int e = __ldg(a.in.fx + (size_t)nb[d] * Ls + s), ep = fx_half<0>(e), em = fx_half<1>(e);
+                const int ab = ep == FX_ZERO || em == FX_ZERO ? 0 : min(max(ep - em, -63), 63);   // zeros need no shift
+                above |= (uint64_t)(uint32_t)(ab & 0xff) << (8 * d);
+            }
+        }
         const int4 *u = GL ? a.gauge_fx + (size_t)site * 72 : sm.u + j * 72;
 #pragma unroll 1
         for (int d = 0; d < 8; ++d) {
             longlong2 Hx[3], Hy[3], Qx[3], Qy[3];
             asm volatile("cp.async.wait_group 0;" ::: "memory");
+            if (above) fx_even_halves(slot, nt, (int8_t)(above >> (8 * d)));
             {
                 longlong2 v[12];
 #pragma unroll
@@ -230,7 +255,7 @@ __global__ void __launch_bounds__(128, 4) hop_fx_kernel(const HopArgs a)
     }
     __syncthreads();   // the slots become the tile
     if (active) {
-        if (mark >= FX_RAW) {
+        if (raw) {
             double2 o[12];
             fx_hop_raw<DAG>(a.in, a.nbr + (size_t)site * 8,
                             reinterpret_cast<const double *>(a.gauge) + (size_t)site * 8 * 18, s, Ls, o);
@@ -238,13 +263,12 @@ __global__ void __launch_bounds__(128, 4) hop_fx_kernel(const HopArgs a)
             fx_put(row, acc, e);
             te[s] = e;
         } else {
-            const bool zero = fx_all_zero(acc);
-            const int w = fx_pairs_width<1>(acc, 0);
+            const int wp = fx_half_width<0>(acc), wm = fx_half_width<1>(acc);
+            te[s] = fx_word(fx_half_zero<0>(acc) ? FX_ZERO : emax - 56 + wp, fx_half_zero<1>(acc) ? FX_ZERO : emax - 56 + wm);
 #pragma unroll
             for (int k = 0; k < 12; ++k)
-                acc[k] = make_longlong2(fx_align(acc[k].x, w, 63 - B), fx_align(acc[k].y, w, 63 - B));
+                acc[k] = make_longlong2(fx_align(acc[k].x, k & 1 ? wm : wp, 63 - B), fx_align(acc[k].y, k & 1 ? wm : wp, 63 - B));
             fx_put(row, acc, 0);
-            te[s] = zero ? FX_ZERO : emax - 56 + w;
         }
     }
     __syncthreads();
@@ -259,7 +283,7 @@ __global__ void __launch_bounds__(128, 4) hop_fx_kernel(const HopArgs a)
             if (a.y.fx) {
                 fx_ld<false>(a.y, (size_t)site, s, Ls, t);
                 e = a.y.fx[(size_t)site * Ls + s];
-                if (e != FX_RAW)
+                if (!fx_is_raw(e))
 #pragma unroll
                     for (int k = 0; k < 12; ++k) t[k] = make_longlong2(t[k].x >> (FX_BITS - B), t[k].y >> (FX_BITS - B));
             } else {

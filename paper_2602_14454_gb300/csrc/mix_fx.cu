@@ -34,7 +34,7 @@ __global__ void __launch_bounds__(128) mix_fx_kernel(const MixArgs a)
         if (a.in.fx) {
             fx_ld<true>(a.in, (size_t)site, s, Ls, t);
             e = a.in.fx[(size_t)site * Ls + s];
-            if (e != FX_RAW)
+            if (!fx_is_raw(e))
 #pragma unroll
                 for (int k = 0; k < 12; ++k) t[k] = make_longlong2(t[k].x >> (FX_BITS - B), t[k].y >> (FX_BITS - B));
         } else {
