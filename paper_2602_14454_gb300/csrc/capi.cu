@@ -234,7 +234,8 @@ static cudaError_t hop_fx(dwf_ctx *h, bool dag, const HopArgs &a0, cudaStream_t 
 // h_par = (c / 2) H v over the two walls (slices 1 and Ls of the source), v = P_+- b4
 // in `scratch` (source_scratch_bytes); null fields when c_1 = c_Ls = 0, where the
 // source is b4 itself.  The other slices of the source are zero, so its hop takes
-// two slices of fixed-point blocks, not Ls (24^3x48, Ls 8: 725 us against 9461 us).
+// two slices, not Ls (24^3x48, Ls 8, fixed-point blocks: 725 us against 9461 us), in the
+// arithmetic that the FP64 operator has (dwf_ctx::use_fx).
 static size_t half2_bytes(const dwf_ctx *h)
 {
     const size_t v = (field_bytes(DWF_F64, h->Vh, 2) + 255) & ~(size_t)255;
@@ -252,7 +253,7 @@ cudaError_t source_hops(dwf_ctx *h, const void *b4, void *scratch, FieldRef hop2
     FieldRef v[2];
     for (int par = 0; par < 2; ++par) {
         v[par].v = (char *)scratch + par * half;
-        v[par].fx = (int *)((char *)v[par].v + ((field_bytes(DWF_F64, h->Vh, 2) + 255) & ~(size_t)255));
+        if (h->use_fx()) v[par].fx = (int *)((char *)v[par].v + ((field_bytes(DWF_F64, h->Vh, 2) + 255) & ~(size_t)255));
         hop2[par].v = (char *)scratch + (2 + par) * half;
     }
     cudaError_t e = launch_walls((const double *)b4, v[0], v[1], h->eo2lex, h->V, st);
@@ -260,9 +261,16 @@ cudaError_t source_hops(dwf_ctx *h, const void *b4, void *scratch, FieldRef hop2
         HopArgs a = hop_args(h, DWF_F64, par, v[1 - par], hop2[par], MAT_ID);
         a.Ls = 2;
         a.post = h->src_mat;
-        a.post_fx = h->src_fx;
-        a.post_band = 2;
-        e = launch_hop_fx(false, a, st);
+        a.zblock = 0;
+        if (h->use_fx()) {
+            a.post_fx = h->src_fx;
+            a.post_band = 2;
+            e = launch_hop_fx(false, a, st);
+        } else {   // FP64 chosen: its direct kernel (the variants differ in the order of the sums only)
+            a.post_prog = h->src_prog;
+            a.mixmode = 1;
+            e = launch_hop(DWF_F64, false, a, 0, 0, 0, st);
+        }
     }
     h->launches += 3;
     return e;
@@ -508,6 +516,10 @@ static int create_impl(const int dims[4], int Ls, double M0, double mf, const do
         if ((e = cudaMalloc(&h->src_fx, sizeof sx)) != cudaSuccess) return fail(e, "cudaMalloc");
         if ((e = cudaMemcpy(h->src_mat, sm, sizeof sm, cudaMemcpyHostToDevice)) != cudaSuccess) return fail(e, "cudaMemcpy");
         if ((e = cudaMemcpy(h->src_fx, sx, sizeof sx, cudaMemcpyHostToDevice)) != cudaSuccess) return fail(e, "cudaMemcpy");
+        MixProg<double> sp = {};
+        for (int k = 0; k < 4; ++k) sp.d1[k >> 1][k & 1] = 1.0, sp.d2[k >> 1][k & 1] = sm[4 * (k >> 1) + 3 * (k & 1)];
+        if ((e = cudaMalloc(&h->src_prog, sizeof sp)) != cudaSuccess) return fail(e, "cudaMalloc");
+        if ((e = cudaMemcpy(h->src_prog, &sp, sizeof sp, cudaMemcpyHostToDevice)) != cudaSuccess) return fail(e, "cudaMemcpy");
         if ((e = cudaMalloc(&h->mats_fx, mx.size() * sizeof(int4))) != cudaSuccess) return fail(e, "cudaMalloc");
         if ((e = cudaMemcpy(h->mats_fx, mx.data(), mx.size() * sizeof(int4), cudaMemcpyHostToDevice)) != cudaSuccess)
             return fail(e, "cudaMemcpy");
@@ -599,6 +611,7 @@ int dwf_destroy(dwf_handle h)
     if (h->mats_fx) cudaFree(h->mats_fx);
     if (h->src_mat) cudaFree(h->src_mat);
     if (h->src_fx) cudaFree(h->src_fx);
+    if (h->src_prog) cudaFree(h->src_prog);
     for (int k = 0; k < 2; ++k)
         if (h->progs_dev[k]) cudaFree(h->progs_dev[k]);
     if (h->nbr) cudaFree(h->nbr);

@@ -307,9 +307,10 @@ struct dwf_ctx {
     void *mats_dev[3] = {nullptr, nullptr, nullptr};   // double / float / float copies (F16 uses float)
     void *mats_fx = nullptr;                           // int4 [MAT_COUNT][2][Ls][Ls]: fixed-point constants
     const int4 *mat_fx(int id) const { return (const int4 *)mats_fx + (size_t)2 * Ls * Ls * id; }
-    // the source's hop on two slices: c / 2 of rows 1 and Ls, as [2][2][2] doubles and constants
+    // the source's hop on two slices: c / 2 of rows 1 and Ls, as [2][2][2] doubles, constants and a program
     double *src_mat = nullptr;
     int4 *src_fx = nullptr;
+    void *src_prog = nullptr;
     int band_fx(int id) const { return fm.diag[id] ? 2 : (fm.band[id] ? 1 : 0); }
     // the FP64 operator runs on fixed-point blocks unless the caller chose an FP64 hop
     // variant or mixing mode of its own

@@ -313,8 +313,8 @@ __global__ void __launch_bounds__(kLinks) pack_gauge_kernel(const double *U, Dim
 }
 
 // ------------------------------------------------------------------- source
-// The two nonzero slices of P^dag (0, ..., 0, b4) as block fields of two slices:
-// P_+ b4 and P_- b4.  Thread per (lexicographic site, slice).
+// The two nonzero slices of P^dag (0, ..., 0, b4) as FP64 or block fields of two
+// slices: P_+ b4 and P_- b4.  Thread per (lexicographic site, slice).
 __global__ void __launch_bounds__(128) walls_kernel(const double *b4, FieldRef even, FieldRef odd, const int *eo2lex, int V)
 {
     const size_t f = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
@@ -326,9 +326,7 @@ __global__ void __launch_bounds__(128) walls_kernel(const double *b4, FieldRef e
     for (int p = 0; p < 12; ++p)   // pair p: spins 0, 1 (p even, P_+) or 2, 3
         v[p] = (p & 1) == w ? make_double2(c[canon_of_internal(2 * p)], c[canon_of_internal(2 * p + 1)])
                             : make_double2(0.0, 0.0);
-    longlong2 t[12];
-    const int e = fx_pack(v, FX_BITS, t);
-    fx_st(lex == eo2lex[i] ? even : odd, i, w, 2, t, e);
+    fx_store_double(lex == eo2lex[i] ? even : odd, i, w, 2, v);
 }
 
 // The 5D source from the walls' hops h (FP64 fields of two slices, c / 2 applied):

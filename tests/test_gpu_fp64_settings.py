@@ -1,0 +1,36 @@
+"""The FP64 settings of a handle: what the entry points do with them."""
+
+import numpy as np
+import pytest
+import torch
+
+from _util import make_pair, rel, to_gpu, to_np
+from paper_2602_14454_gb300 import dwf, inputs
+
+pytestmark = pytest.mark.gpu
+DIMS, LS = (8, 8, 4, 4), 8
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _built(cuda_ok):
+    from paper_2602_14454_gb300 import build
+    build.build()
+
+
+def pair(**kw):
+    op, ref = make_pair(DIMS, LS, 1.8, 0.03, 1.5, 0.5, "neff", 0.6, seed=3, **kw)
+    return op, ref, to_gpu(ref.to_eo(inputs.gaussian_5d(DIMS, LS, 5), 0))
+
+
+def test_source_follows_the_choice_of_fp64_arithmetic():
+    """Unit links keep colours apart: in FP64 a colour far below the others stays accurate to its own size."""
+    U = np.zeros((4,) + DIMS[::-1] + (3, 3), dtype=np.complex128)
+    U[..., range(3), range(3)] = 1.0
+    op, ref, _ = pair(U=U)
+    b4 = inputs.gaussian_4d(DIMS, 6)
+    b4[..., 1] *= 2.0 ** -80
+    want = ref.source_5d(b4)
+    op.set_hop_config("f64", 0, 0, 0)
+    got = to_np(op.source_5d(to_gpu(b4)))
+    for a in range(3):   # a rounding each of eight directions' sum, diagonal and the two's sum
+        assert rel(got[..., a], want[..., a]) < 1e-15, a
