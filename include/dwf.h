@@ -408,8 +408,9 @@ int dwf_get_sweep(dwf_handle h, int prec, int *zblock);
 /* Autotuner: times every hop configuration (all variants, ns in {1, 2, 4},
  * CTAs of 64 to 256 threads, every available mixing mode) on this handle's lattice with CUDA events on
  * `stream` and keeps the fastest.  cache_path (host string, may be NULL)
- * names a text file of earlier results keyed by device name, lattice, Ls and
- * precision: a hit skips the timing, a miss appends the new result.  Needs
+ * names a text file of earlier results keyed by device name, lattice, Ls,
+ * precision and the library's set of kernels (lines of another set are left
+ * alone): a hit skips the timing, a miss appends the new result.  Needs
  * the gauge field.  Errors: DWF_EINVAL, DWF_ENOGAUGE, DWF_ECUDA. */
 int dwf_autotune(dwf_handle h, int prec, const char *cache_path, void *stream);
 

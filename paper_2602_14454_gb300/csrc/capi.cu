@@ -1218,9 +1218,11 @@ int dwf_autotune(dwf_handle h, int prec, const char *cache_path, void *stream)
     if (!h->has_gauge) return dwf_set_error(DWF_ENOGAUGE, "dwf_set_gauge has not been called");
     cudaDeviceProp prop;
     CK(cudaGetDeviceProperties(&prop, h->device));
+    // Raised whenever a kernel, a candidate or a default changes: earlier results no longer tell the fastest then.
+    constexpr int kKernelSet = 2;
     char key[256];
-    std::snprintf(key, sizeof key, "%s|%dx%dx%dx%d|Ls=%d|prec=%d", prop.name, h->dims[0], h->dims[1], h->dims[2],
-                  h->dims[3], h->Ls, prec);
+    std::snprintf(key, sizeof key, "%s|%dx%dx%dx%d|Ls=%d|prec=%d|set=%d", prop.name, h->dims[0], h->dims[1], h->dims[2],
+                  h->dims[3], h->Ls, prec, kKernelSet);
     for (char *c = key; *c; ++c)
         if (*c == ' ') *c = '_';
     if (cache_path) {

@@ -34,3 +34,17 @@ def test_source_follows_the_choice_of_fp64_arithmetic():
     got = to_np(op.source_5d(to_gpu(b4)))
     for a in range(3):   # a rounding each of eight directions' sum, diagonal and the two's sum
         assert rel(got[..., a], want[..., a]) < 1e-15, a
+
+
+@pytest.mark.parametrize("prec,line", [("f64", "0 1 8 1 100.0"), ("f32", "0 1 8 0 100.0")])
+def test_autotune_does_not_take_lines_of_other_kernel_sets(tmp_path, prec, line):
+    """A line without the kernel set's number, as earlier libraries wrote them, is left alone."""
+    op, _, _ = pair()
+    cache = tmp_path / "tune.txt"
+    key = "%s|%dx%dx%dx%d|Ls=%d|prec=%d" % ((torch.cuda.get_device_name().replace(" ", "_"),) + DIMS + (LS, dwf.PREC[prec]))
+    cache.write_text("%s %s\n" % (key, line))
+    cfg = op.autotune(prec, str(cache))
+    lines = cache.read_text().splitlines()
+    assert len(lines) == 2 and lines[0] == "%s %s" % (key, line) and not lines[1].startswith(key + " ")
+    op2, _, _ = pair()
+    assert op2.autotune(prec, str(cache)) == cfg and len(cache.read_text().splitlines()) == 2   # the new line is taken
