@@ -490,9 +490,10 @@ int dwf_time_hop(dwf_handle h, int prec, int reps, int flush_l2, double *us_per_
 
 /* Timing of one stand-alone fifth-direction mixing launch (out = M in with
  * the even-odd factor M = B A5^-1 of Sec. 2.3, per chirality) on an even
- * field in precision prec with mixing mode `mode` (dwf_set_mix_mode: 0 dense
- * on the CUDA cores, 1 structured, 2 tensor cores: tcgen05 MMAs with the
- * accumulator in tensor memory, FP32/FP16 only); as dwf_time_hop otherwise
+ * field in precision prec with mixing mode `mode` (dwf_set_mix_mode: -1 the
+ * built-in default, for FP64 the fixed-point form; 0 dense on the CUDA cores,
+ * 1 structured, both in FP64 arithmetic for FP64; 2 tensor cores: tcgen05
+ * MMAs with the accumulator in tensor memory, FP32/FP16 only); as dwf_time_hop otherwise
  * (*bytes: the field read once and written once).  The handle's own mixing
  * mode is restored.  Errors: DWF_EINVAL (bad argument, mode unavailable),
  * DWF_ECUDA. */

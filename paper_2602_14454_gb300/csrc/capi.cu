@@ -1309,8 +1309,8 @@ int dwf_time_mix(dwf_handle h, int prec, int mode, int reps, int flush_l2, doubl
 {
     if (!h || reps < 1 || !us || !bytes) return dwf_set_error(DWF_EINVAL, "bad argument");
     if (prec != DWF_F64 && prec != DWF_F32 && prec != DWF_F16) return dwf_set_error(DWF_EINVAL, "bad precision");
-    if (mode < 0 || mode > 2 || (mode == 2 && prec == DWF_F64) || (mode == 1 && !h->fm.structured))
-        return dwf_set_error(DWF_EINVAL, "mode must be 0, 1 (if available) or 2 (FP32/FP16)");
+    if (mode < -1 || mode > 2 || (mode == 2 && prec == DWF_F64) || (mode == 1 && !h->fm.structured))
+        return dwf_set_error(DWF_EINVAL, "mode must be -1, 0, 1 (if available) or 2 (FP32/FP16)");
     cudaStream_t st = (cudaStream_t)stream;
     cudaError_t e = cudaSuccess;
     FieldRef in = h->field("th_in", prec, &e), out = h->field("th_out", prec, &e);
@@ -1325,6 +1325,12 @@ int dwf_time_mix(dwf_handle h, int prec, int mode, int reps, int flush_l2, doubl
     }
     const int saved = h->mixmode[prec];
     h->mixmode[prec] = mode;
+    MixArgs m = mix_args(h, prec, in, out, MAT_M);
+    if (prec == DWF_F64) {   // -1: the default's, fixed-point blocks; 0 and 1: the FP64 kernels
+        m.out = mode < 0 ? h->blocks(out) : out;
+        m.mat_fx = mode < 0 ? h->mat_fx(MAT_M) : nullptr;
+        m.band = mode < 0 ? h->band_fx(MAT_M) : h->fm.band[MAT_M];
+    }
     cudaEvent_t e0, e1;
     CK(cudaEventCreate(&e0));
     CK(cudaEventCreate(&e1));
@@ -1332,7 +1338,10 @@ int dwf_time_mix(dwf_handle h, int prec, int mode, int reps, int flush_l2, doubl
     for (int r = -2; r < reps && e == cudaSuccess; ++r) {
         if (flush_l2) e = cudaMemsetAsync(flush, r & 0xff, flush_bytes, st);
         if (e == cudaSuccess) e = cudaEventRecord(e0, st);
-        if (e == cudaSuccess) e = mix(h, prec, in, out, MAT_M, st);
+        if (e == cudaSuccess) {
+            h->launches += 1;
+            e = m.mat_fx ? launch_mix_fx(m, st) : launch_mix(prec, m, st);
+        }
         if (e == cudaSuccess) e = cudaEventRecord(e1, st);
         if (e == cudaSuccess) e = cudaEventSynchronize(e1);
         float ms = 0;

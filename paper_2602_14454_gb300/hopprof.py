@@ -31,7 +31,7 @@ def main(argv=None):
     ap.add_argument("--mix", type=int, default=None, help="fifth-direction mixing mode")
     ap.add_argument("--sweep", type=int, default=None, help="z-planes per sweep column (0: index order, -2: automatic)")
     ap.add_argument("--iteration", action="store_true", help="time the launches of one CG iteration")
-    ap.add_argument("--time-mix", action="store_true", help="time one stand-alone mixing launch (mode --mix)")
+    ap.add_argument("--time-mix", action="store_true", help="time one stand-alone mixing launch (mode --mix; -1: the default)")
     args = ap.parse_args(argv)
 
     import torch

@@ -36,6 +36,16 @@ def test_source_follows_the_choice_of_fp64_arithmetic():
         assert rel(got[..., a], want[..., a]) < 1e-15, a
 
 
+def test_time_mix_times_the_default():
+    op, _, _ = pair()
+    for mode in (-1, 0, 1):
+        us, nbytes = op.time_mix("f64", mode, reps=2, flush_l2=False)
+        assert us > 0 and nbytes == 2 * 24 * 8 * LS * np.prod(DIMS) / 2
+    assert op.time_mix("f32", -1, reps=2, flush_l2=False)[0] > 0
+    with pytest.raises(dwf.DwfError):
+        op.time_mix("f64", 2, reps=2)
+
+
 @pytest.mark.parametrize("prec,line", [("f64", "0 1 8 1 100.0"), ("f32", "0 1 8 0 100.0")])
 def test_autotune_does_not_take_lines_of_other_kernel_sets(tmp_path, prec, line):
     """A line without the kernel set's number, as earlier libraries wrote them, is left alone."""
