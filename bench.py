@@ -289,7 +289,7 @@ def timed_solves(op, b4, n, **kw):
     return e0.elapsed_time(e1) / 1000.0 / n, s
 
 
-KERNEL_NAMES = {0: "hop_kernel", 3: "hop_sweep_kernel", 4: "hop_block_kernel", 5: "hop_kernel_occ (FP16 projection)",
+KERNEL_NAMES = {-1: "hop_fx_kernel (fixed-point blocks)", 0: "hop_kernel", 3: "hop_sweep_kernel", 4: "hop_block_kernel", 5: "hop_kernel_occ (FP16 projection)",
                 7: "hop_lean_kernel", 9: "hop_wa_kernel (warp-autonomous)",
                 10: "hop_tc_kernel (warp tiles, tcgen05 mixing)"}
 

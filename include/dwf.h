@@ -424,15 +424,21 @@ int dwf_autotune(dwf_handle h, int prec, const char *cache_path, void *stream);
  * two TF32 terms each (FP32 accuracy), the accumulator in tensor memory;
  * inside the hop the mixing of a CTA's tile runs as warp-level TF32 MMAs (the
  * matrix split in two TF32 terms; FP32 fields also split the field, FP16
- * fields do not).  Mode 1 runs in hop variant 9 at Ls 8 and 16 (each lane
- * takes whole chains of one spinor component over the Ls slices from the
+ * fields do not).  Mode 1 runs in hop variant 9 at Ls 8 and 16, in FP32 also
+ * 12 (each lane takes whole chains of one spinor component over the Ls slices from the
  * warp's tile into registers; in FP32/FP16 the CG update and the stand-alone
  * mixing keep the dense form's three-row path for banded matrices), else in
  * the direct variant, which it then selects; mode 2 selects the direct
  * variant (CTAs of at least 32 threads, else the dense form runs) or hop
  * variant 10; the CG update keeps the dense form in mode 2.  -1 restores the
- * default: the structured form for DWF_F64 when it is available, dense for
- * DWF_F32 and DWF_F16.  mode 1 is refused when
+ * default: for DWF_F64 the mixing of the fixed-point hop (of the FP64 kernels,
+ * once a variant is set: structured when available); for DWF_F32 dense, but
+ * structured in the hops that mix with inverses only at Ls 12 and 16, where
+ * hop variant and mode are the defaults; for DWF_F16 dense.
+ * dwf_get_mix_mode answers the mode as resolved: at the default 0, or 1 for
+ * DWF_F64 when the structured form is available.  Setting that answer back
+ * leaves the FP64 default as it is, and is an explicit dense choice (no
+ * structured hops) for DWF_F32.  mode 1 is refused when
  * the handle's parameters make the structured form unavailable
  * (|kappa| = |beta0/alpha0| >= 0.95), mode 2 for prec = DWF_F64; both with
  * DWF_EINVAL, as a NULL handle or pointer and a bad prec or mode. */

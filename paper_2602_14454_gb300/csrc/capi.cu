@@ -52,10 +52,10 @@ int dwf_ctx::mix_mode(int prec) const
     const int m = mixmode[prec];
     if (m == 1) return fm.structured ? 1 : 0;
     if (m == 2) return prec == DWF_F64 ? 0 : 2;
-    // default: the structured form in FP64, where the FP64 pipe bounds the hop
-    // (measured 2014 us vs 2217 us at 16^3x32, Ls 16); dense elsewhere (in FP32 the
-    // structured chains of the warp-autonomous hop are 3-4 % faster for K_a and K_c
-    // at 32^3x64 but slower for the banded K_d and the CG update)
+    // default of the FP64 kernels: the structured form, as the FP64 pipe bounds their hop
+    // (measured 2014 us vs 2217 us at 16^3x32, Ls 16); the FP64 default itself mixes on
+    // blocks (use_fx).  Dense elsewhere; which FP32 hops take chains by default instead
+    // is hop_programs' choice.
     if (m < 0 && prec == DWF_F64 && fm.structured) return 1;
     return 0;
 }
@@ -1206,6 +1206,11 @@ int dwf_get_mix_mode(dwf_handle h, int prec, int *mode)
 int dwf_get_hop_config(dwf_handle h, int prec, int *variant, int *ns, int *sb)
 {
     if (!h || prec < 0 || prec > 2 || !variant || !ns || !sb) return dwf_set_error(DWF_EINVAL, "bad argument");
+    if (prec == DWF_F64 && h->use_fx()) {   // no variant has its number: -1 sets it again
+        *variant = -1;
+        *ns = *sb = 0;
+        return DWF_OK;
+    }
     *variant = h->hop_var[prec] >= 0 ? h->hop_var[prec] : hop_default_variant(prec);
     *ns = h->hop_ns[prec] ? h->hop_ns[prec] : hop_default_ns(prec, h->Ls);
     *sb = h->hop_sb[prec] ? h->hop_sb[prec] : hop_default_sb(prec, h->Ls, *ns);

@@ -24,7 +24,8 @@ cudaError_t launch_hop_fx(bool dag, const HopArgs &a, cudaStream_t st)
 // 586 / 8755 us), FP16 variant 5 (84.7 / 1183 us; variant 9: 87.8 / 1372 us).
 // Variant 9 takes dense mixing (FP32 any Ls; FP16 Ls dividing 32 and a multiple of
 // 4) or chains (Ls 8 and 16, FP32 also 12); otherwise the default is variant 0 (FP32)
-// or 5.  FP64 answers 0 here: its default is the fixed-point hop (launch_hop_fx).
+// or 5.  FP64 answers 0 here, its variant where the caller left the fixed-point default
+// (dwf_ctx::use_fx, launch_hop_fx) without naming one.
 int hop_default_variant(int prec) { return prec == DWF_F16 ? 5 : (prec == DWF_F32 ? 9 : 0); }
 
 int hop_default_ns(int prec, int Ls)

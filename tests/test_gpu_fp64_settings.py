@@ -22,6 +22,28 @@ def pair(**kw):
     return op, ref, to_gpu(ref.to_eo(inputs.gaussian_5d(DIMS, LS, 5), 0))
 
 
+def test_reading_and_setting_back_changes_nothing():
+    op, _, x = pair()
+    want = to_np(op.apply(x, op="eo", prec="f64"))
+    op.set_mix_mode("f64", op.mix_mode("f64"))
+    assert np.array_equal(to_np(op.apply(x, op="eo", prec="f64")), want)
+    op.set_hop_config("f64", *op.hop_config("f64"))
+    assert np.array_equal(to_np(op.apply(x, op="eo", prec="f64")), want)
+    op.set_hop_config("f64", 0, 1, 4)   # a choice of the FP64 kernels is reported as set
+    assert op.hop_config("f64") == (0, 1, 4)
+
+
+def test_reading_and_setting_back_with_varying_coefficients():
+    """The resolved mixing mode is 0 here: the structured form needs constant coefficients."""
+    b, c = np.linspace(1.0, 2.0, LS), np.linspace(0.2, 0.6, LS)
+    op = dwf.Operator(DIMS, LS, 1.8, 0.05, list(b), list(c))
+    op.set_gauge(to_gpu(inputs.random_links(DIMS, 0.3, 4)))
+    x = to_gpu(inputs.gaussian_5d(DIMS, LS, 5))
+    want = to_np(op.apply(x, op="full", prec="f64"))
+    op.set_mix_mode("f64", op.mix_mode("f64"))
+    assert np.array_equal(to_np(op.apply(x, op="full", prec="f64")), want)
+
+
 def test_source_follows_the_choice_of_fp64_arithmetic():
     """Unit links keep colours apart: in FP64 a colour far below the others stays accurate to its own size."""
     U = np.zeros((4,) + DIMS[::-1] + (3, 3), dtype=np.complex128)
