@@ -313,11 +313,12 @@ struct dwf_ctx {
     void *src_prog = nullptr;
     int band_fx(int id) const { return fm.diag[id] ? 2 : (fm.band[id] ? 1 : 0); }
     // the FP64 operator runs on fixed-point blocks unless the caller chose an FP64 hop
-    // variant, or a mixing mode other than the one that the default reports (mix_mode):
+    // variant or tile shape (ns, sb), or a mixing mode other than the one that the default reports (mix_mode):
     // setting back what was read changes nothing
     bool use_fx() const
     {
-        return hop_var[DWF_F64] < 0 && (mixmode[DWF_F64] < 0 || mixmode[DWF_F64] == (fm.structured ? 1 : 0));
+        return hop_var[DWF_F64] < 0 && !hop_ns[DWF_F64] && !hop_sb[DWF_F64] &&
+               (mixmode[DWF_F64] < 0 || mixmode[DWF_F64] == (fm.structured ? 1 : 0));
     }
     void *progs_dev[2] = {nullptr, nullptr};           // MixProg<double>[MAT_COUNT], MixProg<float>[MAT_COUNT]
     int mixmode[3] = {-1, -1, -1};    // fifth-direction mixing per precision: 0 dense, 1 structured, 2 tensor cores, -1 default

@@ -44,6 +44,15 @@ def test_reading_and_setting_back_with_varying_coefficients():
     assert np.array_equal(to_np(op.apply(x, op="full", prec="f64")), want)
 
 
+@pytest.mark.parametrize("ns,sb", [(2, 0), (1, 8), (0, 5)])
+def test_a_tile_shape_selects_the_kernels_that_take_it(ns, sb):
+    op, _, x = pair()
+    op.set_hop_config("f64", -1, ns, sb)
+    got = to_np(op.apply(x, op="eo", prec="f64"))
+    op.set_hop_config("f64", 0, ns, sb)
+    assert np.array_equal(got, to_np(op.apply(x, op="eo", prec="f64")))
+
+
 def test_source_follows_the_choice_of_fp64_arithmetic():
     """Unit links keep colours apart: in FP64 a colour far below the others stays accurate to its own size."""
     U = np.zeros((4,) + DIMS[::-1] + (3, 3), dtype=np.complex128)
