@@ -326,7 +326,18 @@ __global__ void __launch_bounds__(128) walls_kernel(const double *b4, FieldRef e
     for (int p = 0; p < 12; ++p)   // pair p: spins 0, 1 (p even, P_+) or 2, 3
         v[p] = (p & 1) == w ? make_double2(c[canon_of_internal(2 * p)], c[canon_of_internal(2 * p + 1)])
                             : make_double2(0.0, 0.0);
-    fx_store_double(lex == eo2lex[i] ? even : odd, i, w, 2, v);
+    const FieldRef &half = lex == eo2lex[i] ? even : odd;
+    if (half.fx) {
+        longlong2 t[12];
+        int e = fx_pack(v, FX_BITS, t);
+        if (!fx_is_raw(e)) {   // the empty half takes the other's exponent: only the hop reads these blocks
+            const int top = max(fx_half<0>(e), fx_half<1>(e));
+            e = fx_word(top, top);
+        }
+        fx_st(half, i, w, 2, t, e);
+    } else {
+        st_pairs<DWF_F64>(half, i, w, 2, v);
+    }
 }
 
 // The 5D source from the walls' hops h (FP64 fields of two slices, c / 2 applied):
