@@ -374,10 +374,11 @@ long long dwf_launch_count(dwf_handle h);
  * in two TF32 terms, FP32 accumulators in tensor memory), the epilogue reads
  * them back row by row (ns and sb must be 0).  ns: slices per thread for the
  * other variants (1, 2 when it divides Ls, 4 for variant 5); sb: sites per
- * CTA.  -1 / 0 select the built-in defaults (FP32: variant 9 where it
- * applies, else 0; FP16: 5; FP64: a hop on 59-bit fixed-point blocks, for
- * which dwf_get_hop_config answers 0; any variant or mixing mode chosen for
- * FP64 selects the FP64 arithmetic instead).  Variants differ only in the order
+ * CTA.  -1 / 0 select the built-in defaults (FP32: variant 9; FP16: 5, and
+ * 9 for one hop of the CG iteration at Ls 8 and 16; FP64: a hop on 59-bit
+ * fixed-point blocks, for which dwf_get_hop_config answers -1, 0, 0; any
+ * variant, ns or sb, or a mixing mode other than the default's, chosen for
+ * FP64 selects FP64 arithmetic instead).  Variants differ only in the order
  * of the sums, except 5 (FP16 rounding of the projection), 10 (products of the
  * TF32 terms) and the FP64 default, whose errors are relative to the largest
  * entry of each (site, s, chirality) and of each link: in the norm of those not
@@ -389,7 +390,8 @@ long long dwf_launch_count(dwf_handle h);
 int dwf_set_hop_config(dwf_handle h, int prec, int variant, int ns, int sb);
 int dwf_get_hop_config(dwf_handle h, int prec, int *variant, int *ns, int *sb);
 
-/* Sweep order of the hop kernels in precision prec (variants 0, 5, 9 and 10):
+/* Sweep order of the hop kernels in precision prec (variants 0, 5, 9 and 10 and
+ * the FP64 default; index order where a tile of sites would straddle two runs):
  * the sites of one parity are taken in columns of zblock z-planes, each column
  * t-slice by t-slice, so that the two reads of a site as the -t and +t
  * neighbour of others lie 2 zblock (Lx/2) Ly sites apart and the field between

@@ -171,7 +171,8 @@ __global__ void __launch_bounds__(128, 4) hop_fx_kernel(const HopArgs a)
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int Ls = LS ? LS : a.Ls, SB = LS ? 128 / LS : (int)blockDim.y, s = threadIdx.x, j = threadIdx.y;
     const int tid = j * Ls + s, nt = Ls * SB, B = fx_mix_bits(Ls);
-    const int site0 = blockIdx.x * SB, site = site0 + j;
+    // in a sweep every CTA is full (hop_fx_launch_ls); the two-slice source has none
+    const int site0 = LS == 2 ? blockIdx.x * SB : sweep_site(a, blockIdx.x * SB), site = site0 + j;
     const bool active = site < a.Vh;
     FxSmem sm;
     constexpr bool GL = fx_global_links(LS);
@@ -357,7 +358,9 @@ cudaError_t hop_fx_launch_ls(const HopArgs &a, cudaStream_t st)
     cudaError_t e = smem_optin(hop_fx_kernel<DAG, LS>, 200 * 1024, optin);
     if (e != cudaSuccess) return e;
     const int SB = 128 / a.Ls;
-    hop_fx_kernel<DAG, LS><<<(a.Vh + SB - 1) / SB, dim3(a.Ls, SB), fx_smem_bytes(a.Ls, SB), st>>>(a);
+    HopArgs b = a;
+    if (b.zblock > 0 && (b.zblock * b.ext[0] * b.ext[1]) % SB) b.zblock = 0;   // a CTA would straddle two runs
+    hop_fx_kernel<DAG, LS><<<(a.Vh + SB - 1) / SB, dim3(a.Ls, SB), fx_smem_bytes(a.Ls, SB), st>>>(b);
     return cudaGetLastError();
 }
 

@@ -389,23 +389,6 @@ __device__ __forceinline__ void gather8(typename Tr<P>::pair (*acc)[12], const H
     }
 }
 
-// Sweep order: sweep position p -> site index.  With a.zblock = Bz (0 < Bz <
-// Lz) the lattice is swept in columns of Bz z-planes, each column t-slice by
-// t-slice: site = r + A (z + Lz t), A = (Lx/2) Ly sites of one parity per
-// z-plane, z = column Bz + zl, p = column (Lt Bz A) + t (Bz A) + zl A + r.  A
-// site's -t and +t neighbours are then read 2 Bz A positions apart instead of
-// 2 Lz A, which keeps the field between the two reads within L2 once a whole
-// t-slice no longer fits; only the z-planes bordering a column are read twice
-// from DRAM.  Consecutive positions stay consecutive sites inside a run of Bz A.
-__device__ __forceinline__ int sweep_site(const HopArgs &a, int p)
-{
-    const int Bz = a.zblock;
-    if (Bz <= 0) return p;
-    const int A = a.ext[0] * a.ext[1], plane = Bz * A, col = plane * a.ext[3];
-    const int c = p / col, q = p - c * col, t = q / plane;
-    return q - t * plane + A * (c * Bz + a.ext[2] * t);
-}
-
 // One tile of SB sites: blockDim = (Ls/NS, SB), site = u SB + threadIdx.y
 // (in the sweep order above when a tile never straddles a run of Bz A sites).
 // The norm reduction runs over the nb_red tiles that share a.red.

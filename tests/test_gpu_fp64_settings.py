@@ -53,6 +53,22 @@ def test_a_tile_shape_selects_the_kernels_that_take_it(ns, sb):
     assert np.array_equal(got, to_np(op.apply(x, op="eo", prec="f64")))
 
 
+@pytest.mark.parametrize("Ls", [8, 10])   # 16 sites to a CTA: half a run of 32; 12 sites straddle runs (index order then)
+def test_sweep_order_of_the_default(Ls):
+    dims = (8, 8, 8, 4)
+    op, ref = make_pair(dims, Ls, 1.8, 0.1, 1.5, 0.5, "neff", 0.6, seed=3)
+    x = to_gpu(ref.to_eo(inputs.gaussian_5d(dims, Ls, 5), 0))
+    b5 = op.source_5d(to_gpu(inputs.gaussian_4d(dims, 6)))
+    want, x5 = to_np(op.apply(x, op="eo", prec="f64")), to_np(op.solve(b5, inner_prec="f64", tol=1e-10)[0])
+    op.set_sweep("f64", 2)
+    assert np.array_equal(to_np(op.apply(x, op="eo", prec="f64")), want)
+    swept, st = op.solve(b5, inner_prec="f64", tol=1e-10)
+    swept = to_np(swept)
+    assert st["true_residual"] < 1e-10 and rel(swept, x5) < 1e-8
+    # the order of the norms' partial sums, and with it the last bits, follows the sweep
+    assert np.array_equal(swept, x5) == (Ls == 10)
+
+
 def test_source_follows_the_choice_of_fp64_arithmetic():
     """Unit links keep colours apart: in FP64 a colour far below the others stays accurate to its own size."""
     U = np.zeros((4,) + DIMS[::-1] + (3, 3), dtype=np.complex128)
