@@ -435,8 +435,8 @@ int dwf_autotune(dwf_handle h, int prec, const char *cache_path, void *stream);
  * variant 10; the CG update keeps the dense form in mode 2.  -1 restores the
  * default: for DWF_F64 the mixing of the fixed-point hop (of the FP64 kernels,
  * once a variant is set: structured when available); for DWF_F32 dense, but
- * structured in the hops that mix with inverses only at Ls 12 and 16, where
- * hop variant and mode are the defaults; for DWF_F16 dense.
+ * structured in the hops that mix with inverses only at Ls 12 and 16 with
+ * |kappa| <= 0.5, where hop variant and mode are the defaults; for DWF_F16 dense.
  * dwf_get_mix_mode answers the mode as resolved: at the default 0, or 1 for
  * DWF_F64 when the structured form is available.  Setting that answer back
  * leaves the FP64 default as it is, and is an explicit dense choice (no

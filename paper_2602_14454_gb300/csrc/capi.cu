@@ -290,9 +290,13 @@ void source_diagonal(const dwf_ctx *h, double y[2])
 // output.  24^3x48, chains against dense: Ls 16 K_a 372 / 426 us, K_b 533 / 591 us;
 // Ls 12 338 / 380, 472 / 515; at Ls 8 the dense form wins (K_a 190 / 186, K_b
 // 261 / 240).  The banded K_d reads three rows per output and stays dense (449 / 578).
+// For |kappa| up to 0.5 only: kappa's own rounding adds along a chain as
+// 1 / (1 - |kappa|).  Error of the even-odd application against 64 bits, chains / dense:
+// 0.83 to 0.98 for |kappa| from 0.2 to 0.5, 1.34 at 0.6 (Ls 16: 7.1e-8 / 5.3e-8).
 HopArgs hop_programs(dwf_ctx *h, int prec, const HopArgs &a)
 {
     if (prec == DWF_F32 && h->mixmode[prec] < 0 && h->fm.structured && (h->Ls == 12 || h->Ls == 16) &&
+        std::fabs(h->fm.prog[MAT_M].kappa) <= 0.5 &&
         (h->hop_var[prec] < 0 || h->hop_var[prec] == 9) && a.ymode != 2 && !a.rin.v) {
         const HopArgs c = with_programs_mode(h, prec, a, 1);
         if (!c.post_band && !(c.zmat && c.z_band)) return c;
