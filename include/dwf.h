@@ -202,8 +202,8 @@ int dwf_apply_dag(dwf_handle h, int op, int prec, const void *in, void *out, voi
 
 /* b5 = (-D_-) P^dag (0, ..., 0, b4)^T  (Sec. 2.3, with D_- = diag_s(c D_W - 1)):
  * b5(s=1) = (1 - c D_W) P_+ b4, b5(s=Ls) = (1 - c D_W) P_- b4, zero elsewhere.
- * b4 is a 4D field, b5 a 5D field (device, caller-owned).  FP64, in the
- * arithmetic of the FP64 operator (dwf_set_hop_config).
+ * b4 is a 4D field, b5 a 5D field (device, caller-owned); b4 may lie in b5.
+ * FP64, in the arithmetic of the FP64 operator (dwf_set_hop_config).
  * Errors: DWF_EINVAL (NULL or unaligned vector), DWF_ENOGAUGE, DWF_ECUDA. */
 int dwf_source_5d(dwf_handle h, const void *b4, void *b5, void *stream);
 

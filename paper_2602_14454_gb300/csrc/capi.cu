@@ -1059,6 +1059,14 @@ int dwf_source_5d(dwf_handle h, const void *b4, void *b5, void *stream)
     cudaError_t e = cudaSuccess;
     void *scratch = h->ws("src_walls", source_scratch_bytes(h), &e);
     if (!scratch) return dwf_cuda_error(e, "workspace");
+    // the walls are written while b4 is read, so a b4 inside b5 (a slice of it) is read from a copy
+    const size_t n4 = (size_t)h->V * 24 * sizeof(double);
+    if ((const char *)b4 < (const char *)b5 + n4 * h->Ls && (const char *)b5 < (const char *)b4 + n4) {
+        void *copy = h->ws("src_b4", n4, &e);
+        if (!copy) return dwf_cuda_error(e, "workspace");
+        CK(cudaMemcpyAsync(copy, b4, n4, cudaMemcpyDeviceToDevice, st));
+        b4 = copy;
+    }
     FieldRef hop2[2];
     double y[2];
     CK(source_hops(h, b4, scratch, hop2, st));
