@@ -287,7 +287,7 @@ void source_diagonal(const dwf_ctx *h, double y[2])
 // variant at their defaults, the hops that mix with inverses only (K_a, K_b, K_c of the
 // CG iteration) take the structured mixing by register chains at Ls 12 and 16: it reads every tile
 // element once where the dense form reads the site's tile and a matrix row per
-// output.  24^3x48, chains against dense: Ls 16 K_a 372 / 426 us, K_b 533 / 591 us;
+// output.  24^3x48, chains against dense (Ls a run-time value then): Ls 16 K_a 372 / 426 us, K_b 533 / 591 us;
 // Ls 12 338 / 380, 472 / 515; at Ls 8 the dense form wins (K_a 190 / 186, K_b
 // 261 / 240).  The banded K_d reads three rows per output and stays dense (449 / 578).
 // For |kappa| up to 0.5 only: kappa's own rounding adds along a chain as
@@ -1279,7 +1279,7 @@ int dwf_autotune(dwf_handle h, int prec, const char *cache_path, void *stream)
                 if (mix == 1 && !h->fm.structured) continue;
                 if (mix == 2 && prec == DWF_F64) continue;
                 if (var == 1 || var == 2 || var == 6 || var == 8) continue;   // numbers not in use
-                if (mix != 0 && var != 0) continue;   // those mixings exist in the direct variant only
+                if (mix != 0 && var != 0) continue;   // variant 9's chains: the default takes them where they win
                 if (var == 5 && prec != DWF_F16) continue;
                 if ((var == 7 || var == 9) && prec == DWF_F64) continue;
                 if (var == 7 && (ns != 1 || h->Ls % 4 != 0)) continue;

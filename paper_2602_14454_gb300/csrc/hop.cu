@@ -18,7 +18,7 @@ cudaError_t launch_hop_fx(bool dag, const HopArgs &a, cudaStream_t st)
     return dag ? hop_fx_launch<true>(a, st) : hop_fx_launch<false>(a, st);
 }
 
-// Defaults from the sweeps on GB300 at 16^3x32 and 32^3x64, Ls 16: FP32 the
+// Defaults from the sweeps on GB300 at 16^3x32 and 32^3x64, Ls 16 (dense mixing): FP32 the
 // warp-autonomous variant 9 (83.7 / 1446 us per hop against 102.4 / 1519 us for
 // the direct variant 0; the whole FP32 CG iteration 475 / 7897 us against
 // 586 / 8755 us), FP16 variant 5 (84.7 / 1183 us; variant 9: 87.8 / 1372 us).
@@ -83,7 +83,8 @@ cudaError_t launch_hop(int prec, bool dag, const HopArgs &a, int var, int NS, in
         NS = 2;
         SB = 4;
     }
-    // variants 7 and 9 need FP32/FP16 fields and dense mixing (9 also Ls dividing 32), else the default
+    // variant 7 needs FP32/FP16 fields, dense mixing and Ls a multiple of 4; variant 9 dense mixing (FP32 any
+    // Ls, FP16 Ls dividing 32 and a multiple of 4) or chains; else variant 5 (FP16) or 0
     const bool v_ok = prec != DWF_F64 && a.mixmode == 0 && a.Ls % 4 == 0;
     const bool v9_ok = prec != DWF_F64 &&
                        ((a.mixmode == 0 && (prec == DWF_F32 || (a.Ls % 4 == 0 && 32 % a.Ls == 0))) ||

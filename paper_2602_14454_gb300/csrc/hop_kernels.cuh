@@ -1330,8 +1330,8 @@ __device__ __forceinline__ void wa_issue_links(const void *gauge, int site0, int
 // the fields exceed L2).
 // bid of nb: this CTA among those that work on a's lattice.
 // LS: Ls, or 0 for any (dense mixing only).  A fixed Ls takes the address arithmetic
-// out of the loops and the spills with it: 24^3x48 K_a 338 us instead of 360 (Ls 16),
-// 307 instead of 328 (Ls 12), the dense hop 397 / 425 and 345 / 377.
+// out of the loops (spills are 20 bytes or fewer either way): 24^3x48 K_a 338 us instead
+// of 360 (Ls 16), 307 instead of 328 (Ls 12), the dense hop 397 / 425 and 345 / 377.
 template <int P, bool DAG, int MIX, int LS>
 __device__ __forceinline__ void hop_wa_body(const HopArgs &a, int bid, int nb)
 {
@@ -2045,8 +2045,8 @@ cudaError_t launch_pd(const HopArgs &a, int var, int NS, int SB, cudaStream_t st
         SB = 4;
     }
 
-    // variant 9: warp-autonomous (FP32 and FP16 fields, dense mixing, Ls dividing 32 and a
-    // multiple of 4); SB = warps per CTA, NS selects the register budget (1: 5 CTAs of 4
+    // variant 9: warp-autonomous (dense mixing: FP32 any Ls, FP16 Ls dividing 32 and a multiple
+    // of 4; chains below); SB = warps per CTA, NS selects the register budget (1: 5 CTAs of 4
     // warps per SM, 2: 4)
     if constexpr (P != DWF_F64) {
         if (var == 9 && a.mixmode == 0 && (P == DWF_F32 || (32 % a.Ls == 0 && a.Ls % 4 == 0))) {
