@@ -18,7 +18,8 @@
 // 1987 us on the FP64 pipe (485 us with one exponent for both halves of a block).  In
 // an earlier form of 502 us (links made into limbs here) the eight directions took
 // about 267 us and the mixing about 155 us, bound by its shared-memory reads.  All
-// forms use 128 registers and spill 250 to 432 bytes a thread.
+// forms use 128 registers; their spills (250 to 490 bytes a thread) lie on paths that are
+// seldom taken: 0.2 % of the executed instructions access local memory.
 #pragma once
 
 #include "fx_fields.cuh"   // before stencil.cuh: its templates take the integer pairs
