@@ -162,7 +162,8 @@ class Extended:
 @pytest.mark.parametrize("dims,Ls,b,c,form", [((4, 4, 4, 4), 8, 1.0, 0.0, "standard"), ((4, 4, 2, 6), 16, 1.5, 0.5, "neff"),
                                               ((4, 4, 4, 4), 12, 1.0, 1.0, "standard"), ((6, 4, 4, 4), 10, 1.5, 0.5, "neff")])
 def test_error_not_above_fp64(dims, Ls, b, c, form):
-    """In the norm, the default's error is not above that of the FP64 kernels (whole matrix, even-odd matrix, source)."""
+    """The default's error is not above that of the FP64 kernels: in the norm (whole matrix, even-odd matrix, source),
+    and on these fields entry by entry (median, 90 % and 99 % of the reals' relative errors; the source holds zeros)."""
     par = (1.8, 0.02, b, c, form, 0.5)
     U = inputs.random_links(dims, 0.3, 11)
     op, _ = make_pair(dims, Ls, *par, U=U)
@@ -173,9 +174,13 @@ def test_error_not_above_fp64(dims, Ls, b, c, form):
              "eo": (lambda: op.apply(to_gpu(xe), op="eo", prec="f64"), D.half(D.eo(x.astype(np.clongdouble) * D.even))),
              "source": (lambda: op.source_5d(to_gpu(b4)), D.source(b4.astype(np.clongdouble), Ls))}
     for name, (call, want) in cases.items():
-        err = []
+        err, entries = [], []
         for got in both(op, call):
             d = got.astype(np.clongdouble) - want
+            if name != "source":
+                r = np.concatenate([abs(d.real / want.real).ravel(), abs(d.imag / want.imag).ravel()]).astype(float)
+                entries.append(np.quantile(r, (0.5, 0.9, 0.99)))
             err.append(float(np.sqrt((abs(d) ** 2).sum() / (abs(want) ** 2).sum())))
         print(name, dims, Ls, "default %.3g, FP64 %.3g" % tuple(err))
         assert err[0] <= err[1], name
+        assert not entries or (entries[0] <= entries[1]).all(), (name, entries)
